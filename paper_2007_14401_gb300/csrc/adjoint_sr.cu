@@ -20,6 +20,7 @@
 #include "dual.cuh"
 #include "gcb_internal.h"
 #include "adjoint_rev.cuh"
+#include "gca_lean.cuh"
 #include "push_sr.cuh"
 
 // Code size of the reverse kernel: its per-point pieces (gather + frame,
@@ -163,8 +164,21 @@ __device__ __forceinline__ void load_pos(const AdjArgs<T> &a, int64_t i, int d, 
     } else {
         const double x = ((const double *)a.x[d])[i];
         fin = fin && isfinite(x);
-        split_pos_f64<T>(x, (double)a.g.dx[d], 1.0 / (double)a.g.dx[d], (double)(a.g.n[d] - 1), ib, l);
+        split_pos_f64<T>(x, (double)a.g.dx[d], 1.0 / (double)a.g.dx[d], a.g.n[d] - 1, ib, l);
     }
+}
+
+// The forward step as the forward run takes it (push_step_f64,
+// push_step_adj_f32).
+template <typename T, typename Gth>
+__device__ __forceinline__ bool replay_step(const Gth &gth, const StepPar<T> &s, const int ib[2],
+                                            const T l[2], const T dxp[2], const FieldPt<T, 2> &F0,
+                                            T u[3], T disp[2], int &iters, bool &nonconv)
+{
+    if constexpr (sizeof(T) == 8)
+        return gca_step_lean<T, 2, 2>(gth, s, ib, l, dxp, F0, u, disp, iters, nonconv);
+    else
+        return gca_step<T, 2, 2>(gth, s, ib, l, dxp, F0, u, disp, iters, nonconv);
 }
 
 template <typename T, int N>
@@ -194,6 +208,7 @@ __global__ void __launch_bounds__(TPB) k_adjoint_sr(const AdjArgs<T> a)
         // plain replay: the switch, the branch and the iteration count
         StepPar<T> sp = a.sp;
         sp.qm = a.qm[(fl >> GCB_SPECIES_SHIFT) & 3];
+        sp.cq = sp.c / sp.qm;
         FieldPt<T, 2> F0;
         gather<T, 2, 2>(a.g, ib, l, F0);
         const T Q = fabs(sp.qm);
@@ -208,7 +223,7 @@ __global__ void __launch_bounds__(TPB) k_adjoint_sr(const AdjArgs<T> a)
         if (S == 0) {
             T uu[3] = {u[0], u[1], u[2]}, disp[2];
             bool ncv;
-            gca = gca_step<T, 2, 2>(PlainGather<T, 2, 2>{a.g}, sp, ib, l, dxp, F0, uu, disp, iters, ncv);
+            gca = replay_step(PlainGather<T, 2, 2>{a.g}, sp, ib, l, dxp, F0, uu, disp, iters, ncv);
         }
         const int ngather = gca ? iters + 2 : 1;
         if (ngather > MAXG) continue;    // excluded by the host's iteration-cap check
@@ -643,6 +658,7 @@ __global__ void __launch_bounds__(TPB, RevBlocks<T>::n) k_adjoint_rev(const AdjA
 
         StepPar<T> sp = a.sp;
         sp.qm = a.qm[(fl >> GCB_SPECIES_SHIFT) & 3];
+        sp.cq = sp.c / sp.qm;
         FieldPt<T, 2> F0;
         gather<T, 2, 2>(a.g, ib, l, F0);
         fc.store(0, F0);
@@ -659,7 +675,7 @@ __global__ void __launch_bounds__(TPB, RevBlocks<T>::n) k_adjoint_rev(const AdjA
             T uu[3] = {u[0], u[1], u[2]}, disp[2];
             bool ncv;
             int cnt = 0;
-            gca = gca_step<T, 2, 2>(RecGather<T>{a.g, pts, &cnt, fc}, sp, ib, l, dxp, F0, uu, disp, K, ncv);
+            gca = replay_step(RecGather<T>{a.g, pts, &cnt, fc}, sp, ib, l, dxp, F0, uu, disp, K, ncv);
             gca = gca && cnt == K + 1 && cnt <= MAXG;
         }
         T li[NS];

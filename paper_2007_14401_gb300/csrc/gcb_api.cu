@@ -862,7 +862,8 @@ gcb_status gcb_push_sr_ckpt(const gcb_particles *p, const gcb_grid *g, const gcb
     if (p->n > 0) {
         const bool fp64 = p->mom_dtype == GCB_F64;
         auto step = [&](const gcb_particles *in) {
-            return fp64 ? push_step_f64(p, in, g, &prm, st, stats) : push_step_f32(p, in, g, &prm, st, stats);
+            return fp64 ? push_step_f64(p, in, g, &prm, st, stats)
+                        : push_step_adj_f32(p, in, g, &prm, st, stats);
         };
         for (int c = 0; c < L.nck; ++c) {
             const gcb_particles *in = p;
@@ -937,7 +938,8 @@ gcb_status gcb_adjoint_sr(const gcb_particles *p0, const gcb_grid *g, const gcb_
     if (p0->n == 0) return GCB_OK;
     const bool fp64 = p0->mom_dtype == GCB_F64;
     auto step = [&](const gcb_particles *out, const gcb_particles *in) {
-        return fp64 ? push_step_f64(out, in, g, &prm, st, stats) : push_step_f32(out, in, g, &prm, st, stats);
+        return fp64 ? push_step_f64(out, in, g, &prm, st, stats)
+                    : push_step_adj_f32(out, in, g, &prm, st, stats);
     };
     gcb_particles tA = state_view(p0, nd, tmp), tB = state_view(p0, nd, tmp + S);
     if (!have_ckpt) {

@@ -15,6 +15,8 @@
 #include <climits>
 #include <type_traits>
 
+#include "real64.cuh"
+
 namespace gcb {
 
 template <typename R>
@@ -78,6 +80,24 @@ __device__ __forceinline__ void cell_of(const DevGrid<R> &g, int d, int ib, R l,
     t = s - c;
     c = fmin(fmax(c, -g.nR[d]), g.nR[d]);
     int i = ib + (int)c;
+    i += i < 0 ? n : 0;
+    i -= i >= n ? n : 0;
+    int j = i + 1;
+    j -= j >= n ? n : 0;
+    i0 = i;
+    i1 = j;
+}
+
+// FP64: the floor and its clamp without FP64 comparisons and conversions.
+template <>
+__device__ __forceinline__ void cell_of<double>(const DevGrid<double> &g, int d, int ib, double l,
+                                                double &t, int &i0, int &i1)
+{
+    const int n = g.n[d];
+    const double s = l * g.inv_dx[d];
+    int k;
+    t = s - floor64(s, n, k);
+    int i = ib + k;
     i += i < 0 ? n : 0;
     i -= i >= n ? n : 0;
     int j = i + 1;
@@ -350,6 +370,74 @@ __device__ __forceinline__ void gather_cached(const DevGrid<float> &g, const int
     interp_cell<ND, GM>(g, cr, t, F);
 }
 
+// Gradients of the shape functions left per cell (to be scaled by inv_dx).
+template <typename R, int GM>
+struct RawGrad { static constexpr bool value = sizeof(R) == 8 && GM == 1; };
+
+// FP64 gather with gradients of the shape functions, by linear interpolation
+// along one axis after the other: the differences that a field component's
+// interpolation takes are also its gradient (22 FP64 operations a component in
+// 3D, 8 in 2D, where weights and their derivatives take 32 and 12, and their
+// products 60 and 12 more a gather).  F.dB is left per cell (RawGrad).
+template <int ND>
+__device__ __forceinline__ void gather_dw64(const DevGrid<double> &g, const int ib[ND],
+                                            const double l[ND], FieldPt<double, ND> &F)
+{
+    int i0[ND], i1[ND];
+    double t[ND];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) cell_of(g, d, ib[d], l[d], t[d], i0[d], i1[d]);
+    constexpr int NC = 1 << ND;
+    const double *rp[NC];
+#pragma unroll
+    for (int o = 0; o < NC; ++o) {
+        int node = ((o & 2) ? i1[1] : i0[1]) * g.n[0] + ((o & 1) ? i1[0] : i0[0]);
+        if (ND == 3) node += ((o & 4) ? i1[ND - 1] : i0[ND - 1]) * g.n[1] * g.n[0];
+        rp[o] = g.rec + (size_t)node * g.stride;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {          // components 2q and 2q + 1 of (E, B)
+        double v[NC][2];
+#pragma unroll
+        for (int o = 0; o < NC; ++o) load_chunk(rp[o] + 2 * q, v[o]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = 2 * q + h;
+            double d[NC / 2], w[NC / 2];   // along x: differences and values
+#pragma unroll
+            for (int o = 0; o < NC / 2; ++o) {
+                d[o] = v[2 * o + 1][h] - v[2 * o][h];
+                w[o] = fma(t[0], d[o], v[2 * o][h]);
+            }
+            double e[NC / 4], f[NC / 4];   // then along y
+#pragma unroll
+            for (int o = 0; o < NC / 4; ++o) {
+                e[o] = w[2 * o + 1] - w[2 * o];
+                f[o] = fma(t[1], e[o], w[2 * o]);
+            }
+            double val = f[0], dx, dy = e[0], dz = 0.0;
+            if constexpr (ND == 3) {
+                dz = f[1] - f[0];
+                val = fma(t[2], dz, f[0]);
+            }
+            if (c < 3) {
+                F.E[c] = val;
+                continue;
+            }
+            dx = fma(t[1], d[1] - d[0], d[0]);
+            if constexpr (ND == 3) {
+                dy = fma(t[2], e[1] - e[0], e[0]);
+                const double d1 = fma(t[1], d[3] - d[2], d[2]);
+                dx = fma(t[2], d1 - dx, dx);
+                F.dB[ND - 1][c - 3] = dz;
+            }
+            F.B[c - 3] = val;
+            F.dB[0][c - 3] = dx;
+            F.dB[1][c - 3] = dy;
+        }
+    }
+}
+
 // The gather used by the kernels: packed FP32x2 for float, scalar for double.
 template <typename R, int ND, int GM>
 __device__ __forceinline__ void gather_any(const DevGrid<R> &g, const int ib[ND], const R l[ND],
@@ -569,6 +657,7 @@ __device__ __forceinline__ void make_frame(const FieldPt<R, ND> &F, R c, R inv_c
 template <typename R>
 struct StepPar {
     R c, inv_c2, dt, half_dt, qm;
+    R cq;        // c / qm
     int curvature, mu_mode, max_iter, fixed_iters;
     R tol;
     int phase;   // 1: the gyration phase advances over the step (GCB_PHASE_EVOLVE)
@@ -710,7 +799,8 @@ __device__ __forceinline__ void boris(const R E[3], const R B[3], const StepPar<
 #ifndef GCB_CELL_CACHE_3D
 #define GCB_CELL_CACHE_3D 1
 #endif
-template <typename R, int ND, int GM>
+// RAW: shape-function gradients left per cell (FP64, see RawGrad).
+template <typename R, int ND, int GM, bool RAW = false>
 struct PlainGather {
     static constexpr bool kCellCache =
         sizeof(R) == 4 && (ND == 2 ? GCB_CELL_CACHE_2D : GCB_CELL_CACHE_3D);
@@ -718,7 +808,8 @@ struct PlainGather {
     __device__ __forceinline__ void operator()(const int ib[ND], const R l[ND],
                                                FieldPt<R, ND> &F) const
     {
-        gather_any<R, ND, GM>(g, ib, l, F);
+        if constexpr (RAW) gather_dw64<ND>(g, ib, l, F);
+        else gather_any<R, ND, GM>(g, ib, l, F);
     }
     template <typename C>
     __device__ __forceinline__ void cached(const int ib[ND], const R l[ND], FieldPt<R, ND> &F,

@@ -33,6 +33,8 @@ gcb_status push_step_f64(const gcb_particles *p, const gcb_particles *in, const 
 gcb_status push_step_f32(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
                          const gcb_params *prm, cudaStream_t st, unsigned long long *stats,
                          int nsteps = 1);
+gcb_status push_step_adj_f32(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
+                             const gcb_params *prm, cudaStream_t st, unsigned long long *stats);
 // One unfused step with the mirror terms (push_mir_*.cu).
 gcb_status push_mir_step_f64(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
                              const gcb_params *prm, cudaStream_t st, unsigned long long *stats);

@@ -15,6 +15,7 @@
 // Counters are reduced per block and added atomically to the workspace.
 #pragma once
 
+#include "gca_lean.cuh"
 #include "gcb_device.cuh"
 #include "gcb_internal.h"
 
@@ -97,8 +98,9 @@ struct PushArgs {
     R *dxp[3];
     uint8_t *flags;
     int64_t *pid;             // written only when pidin differs
-    StepPar<R> sp;            // sp.qm is set per particle
-    R qm[4];
+    StepPar<R> sp;            // sp.qm and sp.cq are set per particle
+    R qm[4], cq[4];           // per species: q/m and c/(q/m)
+    double sw[4], f_E2;       // FP64 switch: (f_rho dl |q/m|/c^2)^2 and f_E^2
     R rho_thr;                // f_rho * dl
     R f_E;
     R c2;
@@ -166,11 +168,16 @@ struct PosType<1> { using T = float; };
 // (positions are kept in [0, L); the clamp only matters for positions that
 // rounding put on an edge or for invalid input).
 template <typename R>
-__device__ __forceinline__ void split_pos_f64(double x, double dxd, double inv_dxd, double nmax,
+__device__ __forceinline__ void split_pos_f64(double x, double dxd, double inv_dxd, int nmax,
                                               int &ib, R &l)
 {
-    double fl = fmin(fmax(floor(x * inv_dxd), 0.0), nmax);
-    ib = (int)fl;
+    int k;
+    double fl = floor64(x * inv_dxd, INT_MAX, k);
+    if (k < 0 || k > nmax) {
+        k = k < 0 ? 0 : nmax;
+        fl = (double)k;
+    }
+    ib = k;
     l = (R)fma(-fl, dxd, x);
 }
 __device__ __forceinline__ void split_pos_pair(float h, float lo, float dx, float inv_dx,
@@ -215,15 +222,16 @@ __device__ __forceinline__ void pair_add_wrap(float &h, float &lo, float d, floa
     }
 }
 
+// (comparisons on the bit patterns: x < 0 by its sign, x >= L for x >= 0 as integers)
 __device__ __forceinline__ double wrap_f64(double x, double L)
 {
-    if (x < 0.0) x += L;
-    if (x >= L) x -= L;
+    if (__double_as_longlong(x) < 0) x += L;
+    if (!gt_nonneg(L, x)) x -= L;
     return x;
 }
 
-template <typename R>
-__device__ __forceinline__ bool finite_r(R v) { return isfinite(v); }
+__device__ __forceinline__ bool finite_r(float v) { return isfinite(v); }
+__device__ __forceinline__ bool finite_r(double v) { return finite64(v); }
 
 // ---------------------------------------------------------------------------
 // Current deposition (gcb_push_deposit_sr): the current of a cloud-in-cell
@@ -398,8 +406,9 @@ __device__ __forceinline__ bool deposit_path(const PushArgs<R> &a, const int ib[
 // test-particle mode); every step's arithmetic is the unfused step's.
 // DEP (unfused only): each advanced particle-step also adds its current to a.J.
 // MIR (unfused only): the guiding-center step with the mirror terms.
+// GEN: gca_step_c where gca_lean.cuh would be used (the adjoint's forward run).
 template <typename R, int ND, int PM, int GM, bool FUSE, bool BT = false, bool DEP = false,
-          bool MIR = false>
+          bool MIR = false, bool GEN = false>
 __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) k_push_sr(const PushArgs<R> a)
 {
     static_assert(!(DEP && FUSE), "deposition runs in unfused launches");
@@ -480,7 +489,10 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
         constexpr bool HOIST = GCB_HOIST_HALF && ND == 2;
         FieldPt<R, ND> Fh;          // fields at R^{n-1/2} (HOIST)
         int ib[ND];
-        using Gth = PlainGather<R, ND, GM>;
+        // the step's arrangement: gca_lean.cuh for the simplified frame in FP64
+        // and in FP32 2D, gca_step_c otherwise
+        constexpr bool LEAN = !BT && !GEN && (sizeof(R) == 8 || ND == 2);
+        using Gth = PlainGather<R, ND, GM, LEAN && RawGrad<R, GM>::value>;
         StepRecs<Gth, ND, GM> cr;
         cr.clear();
         if (valid) {
@@ -518,7 +530,7 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
                 for (int d = 0; d < ND; ++d) {
                     if (PM == 0)
                         split_pos_f64<R>((double)xs[d], a.dxd[d], a.inv_dxd[d],
-                                         (double)(a.g.n[d] - 1), ib[d], l[d]);
+                                         a.g.n[d] - 1, ib[d], l[d]);
                     else {
                         float lf;
                         split_pos_pair((float)xs[d], xl[d], (float)a.g.dx[d], (float)a.g.inv_dx[d],
@@ -527,20 +539,28 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
                     }
                 }
                 if constexpr (GCB_SEED_CACHE && Gth::kCellCache) gather_cached<ND, GM>(a.g, ib, l, F, cr);
-                else gather_any<R, ND, GM>(a.g, ib, l, F);
+                else Gth{a.g}(ib, l, F);
                 if constexpr (HOIST) {
                     R ph[ND];
 #pragma unroll
                     for (int d = 0; d < ND; ++d) ph[d] = fma(R(-0.5), dd[d], l[d]);
-                    gather_any<R, ND, GM>(a.g, ib, ph, Fh);
+                    Gth{a.g}(ib, ph, Fh);
                 }
                 // switch S (Sec. 3, Sec. 4.1) in division-free form:
                 // S = 0 iff c^2 Gamma < f_rho dl |q/m| B and |E| < f_E B.
-                R Q = fabs(a.qm[(fl >> GCB_SPECIES_SHIFT) & 3]);
-                R G = sqrt(R(1) + dot3(uu, uu) * a.sp.inv_c2);
-                R Bm = sqrt(dot3(F.B, F.B));
-                R Em = sqrt(dot3(F.E, F.E));
-                int S = (a.c2 * G < a.rho_thr * Q * Bm && Em < a.f_E * Bm) ? 0 : 1;
+                int S;
+                if constexpr (sizeof(R) == 8) {
+                    // squared: no roots (each ~10 FP64 operations)
+                    const double G2 = fma(dot3(uu, uu), a.sp.inv_c2, 1.0);
+                    const double B2 = dot3(F.B, F.B), E2 = dot3(F.E, F.E);
+                    S = (G2 < a.sw[(fl >> GCB_SPECIES_SHIFT) & 3] * B2 && E2 < a.f_E2 * B2) ? 0 : 1;
+                } else {
+                    R Q = fabs(a.qm[(fl >> GCB_SPECIES_SHIFT) & 3]);
+                    R G = sqrt(R(1) + dot3(uu, uu) * a.sp.inv_c2);
+                    R Bm = sqrt(dot3(F.B, F.B));
+                    R Em = sqrt(dot3(F.E, F.E));
+                    S = (a.c2 * G < a.rho_thr * Q * Bm && Em < a.f_E * Bm) ? 0 : 1;
+                }
                 if (a.force == GCB_FORCE_BORIS) S = 1;
                 if (a.force == GCB_FORCE_GCA) S = 0;
                 cls = S;
@@ -680,6 +700,7 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
             const uint8_t f0 = REG ? fl : s_fl[sl];
             StepPar<R> sp = a.sp;
             sp.qm = a.qm[(f0 >> GCB_SPECIES_SHIFT) & 3];
+            sp.cq = a.cq[(f0 >> GCB_SPECIES_SHIFT) & 3];
             R ds[ND], us[3], disp[ND];
 #pragma unroll
             for (int d = 0; d < ND; ++d) ds[d] = REG ? dd[d] : s_d[d][sl];
@@ -690,9 +711,14 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
             bool done = false;
             R vzg = R(0);   // out-of-plane guiding-center velocity of the step (2D DEP)
             if (isg) {
-                done = gca_step_c<R, ND, GM, Gth, BT, MIR>(Gth{a.g}, sp, ib, l, ds, F, us, disp, it,
-                                                      ncv, cr, (HOIST && uni) ? &Fh : nullptr,
-                                                      (DEP && ND == 2) ? &vzg : nullptr);
+                if constexpr (LEAN)
+                    done = gca_step_lean<R, ND, GM, Gth, MIR>(Gth{a.g}, sp, ib, l, ds, F, us, disp,
+                                                              it, ncv, (HOIST && uni) ? &Fh : nullptr,
+                                                              (DEP && ND == 2) ? &vzg : nullptr);
+                else
+                    done = gca_step_c<R, ND, GM, Gth, BT, MIR>(Gth{a.g}, sp, ib, l, ds, F, us, disp, it,
+                                                          ncv, cr, (HOIST && uni) ? &Fh : nullptr,
+                                                          (DEP && ND == 2) ? &vzg : nullptr);
                 if (!done) {
                     fail = true;
                     it = 0;
@@ -701,7 +727,10 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
                     for (int k = 0; k < 3; ++k) us[k] = REG ? uu[k] : s_u[k][sl];
                 }
             }
-            if (!done) boris<R, ND>(F.E, F.B, sp, us, disp);
+            if (!done) {
+                if constexpr (sizeof(R) == 8) boris_lean<ND>(F.E, F.B, sp, us, disp);
+                else boris<R, ND>(F.E, F.B, sp, us, disp);
+            }
             // store: x^{n+1} = x^n + disp (wrapped), dxp = disp
             PosT xn[ND];
             float xln[ND];
@@ -769,7 +798,8 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
                 si += it;
                 mi = max(mi, (unsigned)it);
                 R u2 = dot3(us, us) * sp.inv_c2;
-                ek += (double)(u2 / (R(1) + sqrt(R(1) + u2)));
+                if constexpr (sizeof(R) == 8) ek = fma(u2, rcp64(1.0 + sqrt64(1.0 + u2)), ek);
+                else ek += (double)(u2 / (R(1) + sqrt(R(1) + u2)));
             } else {
                 // not advanced: the input state is kept (copied when the input
                 // is a sorted copy rather than the output arrays themselves;
@@ -904,7 +934,14 @@ static void fill_args(PushArgs<R> &a, const gcb_particles *p, const gcb_particle
     a.sp.max_iter = prm->gca_max_iter;
     a.sp.fixed_iters = prm->gca_fixed_iters;
     a.sp.tol = (R)prm->gca_tol;
-    for (int k = 0; k < 4; ++k) a.qm[k] = (R)prm->qm[k];
+    a.sp.cq = R(0);
+    for (int k = 0; k < 4; ++k) {
+        a.qm[k] = (R)prm->qm[k];
+        a.cq[k] = a.sp.c / a.qm[k];
+        const double w = prm->f_rho * prm->dl * fabs(prm->qm[k]) / (prm->c * prm->c);
+        a.sw[k] = w * w;
+    }
+    a.f_E2 = prm->f_E * prm->f_E;
     a.rho_thr = (R)(prm->f_rho * prm->dl);
     a.f_E = (R)prm->f_E;
     a.c2 = (R)(prm->c * prm->c);
@@ -924,7 +961,7 @@ static void fill_args(PushArgs<R> &a, const gcb_particles *p, const gcb_particle
 }
 
 template <typename R, int ND, int PM, int GM, bool FUSE, bool BT = false, bool DEP = false,
-          bool MIR = false>
+          bool MIR = false, bool GEN = false>
 static gcb_status launch_push(const PushArgs<R> &a, cudaStream_t st)
 {
     static int grid_cache[64] = {0};
@@ -937,7 +974,7 @@ static gcb_status launch_push(const PushArgs<R> &a, cudaStream_t st)
     if (grid == 0) {
         int nsm = 0, occ = 0;
         if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_push_sr<R, ND, PM, GM, FUSE, BT, DEP, MIR>,
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_push_sr<R, ND, PM, GM, FUSE, BT, DEP, MIR, GEN>,
                                                           Tile<R, ND>::n, 0) !=
                 cudaSuccess) {
             set_error("occupancy query failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -950,7 +987,7 @@ static gcb_status launch_push(const PushArgs<R> &a, cudaStream_t st)
     int64_t ntiles = (a.np + TPB - 1) / TPB;
     if (ntiles == 0) return GCB_OK;
     int nb = (int)(ntiles < grid ? ntiles : grid);
-    k_push_sr<R, ND, PM, GM, FUSE, BT, DEP, MIR><<<nb, TPB, 0, st>>>(a);
+    k_push_sr<R, ND, PM, GM, FUSE, BT, DEP, MIR, GEN><<<nb, TPB, 0, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error("kernel launch failed: %s", cudaGetErrorString(e));
