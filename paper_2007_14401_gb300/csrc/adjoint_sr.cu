@@ -755,6 +755,7 @@ gcb_status adjoint_step(const gcb_particles *s, const gcb_grid *g, const gcb_par
         a.g.stride = g->stride;
         for (int d = 0; d < 3; ++d) {
             a.g.n[d] = (int)g->n[d];
+            a.g.nin[d] = g->n[d] <= (1 << 22) ? (int)g->n[d] - 1 : 0;
             a.g.nR[d] = (T)g->n[d];
             a.g.dx[d] = (T)g->dx[d];
             a.g.inv_dx[d] = (T)(1.0 / g->dx[d]);

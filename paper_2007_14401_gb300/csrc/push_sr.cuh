@@ -902,6 +902,7 @@ static void fill_args(PushArgs<R> &a, const gcb_particles *p, const gcb_particle
     a.g.stride = g->stride;
     for (int d = 0; d < 3; ++d) {
         a.g.n[d] = (int)g->n[d];
+        a.g.nin[d] = g->n[d] <= (1 << 22) ? (int)g->n[d] - 1 : 0;
         a.g.nR[d] = (R)g->n[d];
         a.g.dx[d] = (R)g->dx[d];
         a.g.inv_dx[d] = (R)(1.0 / g->dx[d]);
