@@ -1,11 +1,9 @@
 // push_sr.cuh -- one coupled step (Sec. 3.1) over all particles, one kernel.
 //
 // Each block walks tiles of TPB consecutive particles (persistent grid):
-//   phase 1  every thread loads one particle (coalesced SoA loads; the
-//            unfused FP32 2D kernels take it from shared memory, where
-//            asynchronous copies issued during the previous tile put it),
-//            gathers E, B at x^n, evaluates the switch S and stages the
-//            particle in shared memory;
+//   phase 1  every thread loads one particle (coalesced SoA loads), gathers
+//            E, B at x^n, evaluates the switch S and stages the particle in
+//            shared memory;
 //   compact  a warp ballot per branch plus a block prefix over the per-warp
 //            counts orders the tile's slots as [GCA ..., Boris ..., frozen],
 //            so all warps but one run a single branch and GCA lanes run the
@@ -113,7 +111,6 @@ struct PushArgs {
     R dq[4];                  // charge per species
     R jc[3];                  // dx_a / (dt V): J_a per cell of displacement along a
     R jz;                     // 1 / V: 2D J_z per unit v_z and step fraction
-    int pf;                   // the input state is in device memory (GCB_PREFETCH_STATE)
 };
 
 // Particle state is read and written once per step and the field records
@@ -134,28 +131,6 @@ __device__ __forceinline__ void st_state(T *p, T v)
     if constexpr (GCB_STREAM_STATE) __stcs(p, v);
     else *p = v;
 }
-
-// 1: unfused FP32 2D kernels copy the state of the block's next tile into
-// shared memory with asynchronous copies (cp.async) while the current tile
-// is advanced, so that the state's DRAM latency overlaps a tile of
-// arithmetic instead of stalling the tile's first gather (state in device
-// memory only; host-resident state is read directly).  Measured 1.3% faster
-// on the 2D push (2^24 particles); no effect on the 3D push, whose
-// deposition kernels it made spill.
-#ifndef GCB_PREFETCH_STATE
-#define GCB_PREFETCH_STATE 1
-#endif
-template <int B>
-__device__ __forceinline__ void cp_async(void *dst, const void *src)
-{
-    static_assert(B == 4 || B == 8, "4- or 8-byte elements");
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(d), "l"(src), "n"(B)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 template <int PM>
 struct PosType;
@@ -428,15 +403,6 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
     __shared__ int s_wc[2][NWARP];
     __shared__ unsigned long long s_acc[ST_COUNT];
     __shared__ double s_ek;
-    // the state of this block's next tile, copied while the current one is
-    // advanced (two buffers: the copies into one overlap the reads of the other)
-    constexpr bool PF = GCB_PREFETCH_STATE && !FUSE && sizeof(R) == 4 && ND == 2;
-    constexpr int PFN = PF ? TPB : 1;
-    __shared__ PosT s_px[2][ND][PFN];
-    __shared__ float s_pxl[2][PM ? ND : 1][PFN];
-    __shared__ R s_pd[2][ND][PFN];
-    __shared__ R s_pu[2][3][PFN];
-
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid < ST_COUNT) s_acc[tid] = 0ull;
     if (tid == 0) s_ek = 0.0;
@@ -446,38 +412,12 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
     double ek = 0.0;
 
     const int64_t ntiles = (a.np + TPB - 1) / TPB;
-    const bool pf = PF && a.pf;
-    int pb = 0;              // buffer holding the current tile's state
-    uint8_t fl_next = 0;     // the next tile's flag (a plain load, one tile ahead)
-    // copies of particle j's state into buffer b (one commit group per tile)
-    auto prefetch = [&](int b, int64_t j) {
-        if (j < a.np) {
-#pragma unroll
-            for (int d = 0; d < ND; ++d) {
-                cp_async<sizeof(PosT)>(&s_px[b][d][tid], reinterpret_cast<const PosT *>(a.xin[d]) + j);
-                if (PM) cp_async<4>(&s_pxl[b][d][tid], a.xloin[d] + j);
-                cp_async<sizeof(R)>(&s_pd[b][d][tid], a.dxpin[d] + j);
-            }
-#pragma unroll
-            for (int k = 0; k < 3; ++k) cp_async<sizeof(R)>(&s_pu[b][k][tid], a.uin[k] + j);
-            fl_next = ld_state(a.flagsin + j);
-        }
-        cp_async_commit();
-    };
     // tiles strided over the grid: at any moment the blocks of all SMs work
     // on neighbouring tiles, so the field records in use stay few and hot
     // in L2 (one contiguous run of tiles per block measured 48% slower)
-    if (pf) prefetch(0, (int64_t)blockIdx.x * TPB + tid);
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
       const int64_t i = tile * TPB + tid;
       const bool valid = i < a.np;
-      // the next tile's copies go out before this tile's are awaited
-      uint8_t fl_cur = 0;
-      if (pf) {
-          fl_cur = fl_next;
-          prefetch(pb ^ 1, i + (int64_t)gridDim.x * TPB);
-          cp_async_wait<1>();
-      }
       for (int stp = 0; stp < (FUSE ? a.nsteps : 1); ++stp) {
         int cls = 2;
         uint8_t fl = 0;
@@ -499,27 +439,15 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
             const bool from_smem = FUSE && stp > 0;   // the slot holds the previous step's output
             if (!from_smem && a.pidin != a.pid) pid = ld_state(a.pidin + i);
             bool fin = true;
-            if (pf) {
-                fl = fl_cur;
+            fl = from_smem ? s_fl[tid] : ld_state(a.flagsin + i);
 #pragma unroll
-                for (int d = 0; d < ND; ++d) {
-                    xs[d] = s_px[pb][d][tid];
-                    xl[d] = PM ? s_pxl[pb][d][tid] : 0.0f;
-                    dd[d] = s_pd[pb][d][tid];
-                }
-#pragma unroll
-                for (int k = 0; k < 3; ++k) uu[k] = s_pu[pb][k][tid];
-            } else {
-                fl = from_smem ? s_fl[tid] : ld_state(a.flagsin + i);
-#pragma unroll
-                for (int d = 0; d < ND; ++d) {
-                    xs[d] = from_smem ? s_x[d][tid] : ld_state(reinterpret_cast<const PosT *>(a.xin[d]) + i);
-                    xl[d] = PM ? (from_smem ? s_xl[d][tid] : ld_state(a.xloin[d] + i)) : 0.0f;
-                    dd[d] = from_smem ? s_d[d][tid] : ld_state(a.dxpin[d] + i);
-                }
-#pragma unroll
-                for (int k = 0; k < 3; ++k) uu[k] = from_smem ? s_u[k][tid] : ld_state(a.uin[k] + i);
+            for (int d = 0; d < ND; ++d) {
+                xs[d] = from_smem ? s_x[d][tid] : ld_state(reinterpret_cast<const PosT *>(a.xin[d]) + i);
+                xl[d] = PM ? (from_smem ? s_xl[d][tid] : ld_state(a.xloin[d] + i)) : 0.0f;
+                dd[d] = from_smem ? s_d[d][tid] : ld_state(a.dxpin[d] + i);
             }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) uu[k] = from_smem ? s_u[k][tid] : ld_state(a.uin[k] + i);
 #pragma unroll
             for (int d = 0; d < ND; ++d)
                 fin = fin && finite_r(xs[d]) && finite_r(xl[d]) && finite_r(dd[d]);
@@ -844,9 +772,7 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
           for (int k = 0; k < 3; ++k) st_state(a.u[k] + i, s_u[k][tid]);
           st_state(a.flags + i, s_fl[tid]);
       }
-      pb ^= 1;
     }
-    if (pf) cp_async_wait<0>();   // the last (empty) group
 
     // block reduction of the counters
     unsigned vals[9] = {nb, ng, tg, tb, nc, gf, nf, si, mi};
@@ -884,16 +810,6 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
 // ---------------------------------------------------------------------------
 // host side: argument packing and launch
 // ---------------------------------------------------------------------------
-static bool device_memory(const void *ptr)
-{
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice;
-}
-
 template <typename R>
 static void fill_args(PushArgs<R> &a, const gcb_particles *p, const gcb_particles *in,
                       const gcb_grid *g, const gcb_params *prm, unsigned long long *stats)
@@ -949,16 +865,6 @@ static void fill_args(PushArgs<R> &a, const gcb_particles *p, const gcb_particle
     a.force = prm->force;
     a.nsteps = 1;
     a.stats = stats;
-    // the asynchronous copies of the state's next tile read device memory
-    // only; a state in host (or managed) memory is read with plain loads
-    a.pf = 1;
-    for (int d = 0; d < g->ndim; ++d) {
-        const void *arrs[3] = {in->x[d], in->dxp[d], in->pos_mode == GCB_POS_F32PAIR ? in->x_lo[d] : nullptr};
-        for (const void *q : arrs)
-            if (q && !device_memory(q)) a.pf = 0;
-    }
-    for (int k = 0; k < 3; ++k)
-        if (!device_memory(in->u[k])) a.pf = 0;
 }
 
 template <typename R, int ND, int PM, int GM, bool FUSE, bool BT = false, bool DEP = false,
