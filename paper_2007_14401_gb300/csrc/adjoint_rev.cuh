@@ -15,6 +15,52 @@
 namespace gcb {
 namespace rev {
 
+// Reciprocals and reciprocal roots: the approximate instructions in FP32, one
+// Householder step from them in FP64 (real64.cuh).
+__device__ __forceinline__ float rsq_r(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsq_r(double x) { return rsqrt64(x); }
+__device__ __forceinline__ float rcp_r(float x) { return 1.0f / x; }
+__device__ __forceinline__ double rcp_r(double x) { return rcp64(x); }
+
+// The frame as the transposes need it: with 1/|B|, its square, E x B, 1 -
+// v_E^2/c^2, 1/kappa and the unscaled directional derivatives w = (b.grad)B, y =
+// (v_E.grad)B kept.  bgb = w/|B| and vgb = y/|B| are left unprojected: every
+// use is b x (.) or v_E . (.), which annihilates their component along b for
+// any fields, so that the step's derivative does not depend on it.
+template <typename T, int ND>
+struct RFrame {
+    T Bmag, ib, ib2, b[3], x[3], vE[3], om, kappa, ikap, Epar, w[3], y[3], bgb[3], vgb[3];
+
+    __device__ __forceinline__ void make(const FieldPt<T, ND> &F, T c)
+    {
+        const T B2 = dot3(F.B, F.B);
+        ib = rsq_r(B2);
+        Bmag = B2 * ib;
+        ib2 = ib * ib;
+        cross3(F.E, F.B, x);
+        const T cv = c * ib2;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { b[k] = F.B[k] * ib; vE[k] = cv * x[k]; }
+        om = one_minus_beta2<T>(F.E, F.B, B2, c, dot3(x, x) * (ib2 * ib2));
+        kappa = rsq_r(om);
+        ikap = om * kappa;
+        Epar = dot3(F.E, b);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            T sw = b[0] * F.dB[0][j], sy = vE[0] * F.dB[0][j];
+#pragma unroll
+            for (int i = 1; i < ND; ++i) {
+                sw = fma(b[i], F.dB[i][j], sw);
+                sy = fma(vE[i], F.dB[i][j], sy);
+            }
+            w[j] = sw;
+            y[j] = sy;
+            bgb[j] = sw * ib;
+            vgb[j] = sy * ib;
+        }
+    }
+};
+
 template <typename T>
 struct FrameAdj {
     T Bmag, b[3], vE[3], kappa, Epar, bgb[3], vgb[3];
@@ -26,140 +72,126 @@ struct FrameAdj {
     }
 };
 
-// Adjoint of make_frame (with gradients): aF = (d frame / dF)^T af.
+// Adjoint of RFrame::make: aF = (d frame / dF)^T af.
 template <typename T, int ND>
-__device__ __forceinline__ void frame_bwd(const FieldPt<T, ND> &F, T c, T inv_c2,
-                                          const FrameAdj<T> &af, FieldPt<T, ND> &aF)
+__device__ __forceinline__ void frame_bwd(const FieldPt<T, ND> &F, const RFrame<T, ND> &f, T c,
+                                          T inv_c2, const FrameAdj<T> &af, FieldPt<T, ND> &aF)
 {
-    const T B2 = dot3(F.B, F.B);
-    const T Bmag = sqrt(B2);
-    const T ib = T(1) / Bmag;
-    const T ib2 = ib * ib;
-    T b[3], x[3], vE[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) b[k] = F.B[k] * ib;
-    cross3(F.E, F.B, x);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) vE[k] = c * x[k] * ib2;
-    const T beta2 = dot3(vE, vE) * inv_c2;
-    const T om = one_minus_beta2<T>(F.E, F.B, B2, c, beta2);
-    const T kappa = T(1) / sqrt(om);
-    T w[3], y[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        T sw = T(0), sy = T(0);
-#pragma unroll
-        for (int i = 0; i < ND; ++i) {
-            sw = fma(b[i], F.dB[i][j], sw);
-            sy = fma(vE[i], F.dB[i][j], sy);
-        }
-        w[j] = sw;
-        y[j] = sy;
-    }
-    const T bw = dot3(b, w), by = dot3(b, y);
-
     T ab[3], avE[3], aw[3], ay[3];
-    T aib = T(0), abw = T(0), aby = T(0);
-    // bgb_j = (w_j - b_j bw) ib,  vgb_j = (y_j - b_j by) ib
+    // bgb = w ib,  vgb = y ib
+    T aib = dot3(af.bgb, f.w) + dot3(af.vgb, f.y);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        aw[j] = af.bgb[j] * ib;
-        ay[j] = af.vgb[j] * ib;
-        ab[j] = af.b[j] - (af.bgb[j] * bw + af.vgb[j] * by) * ib;
-        abw -= af.bgb[j] * b[j];
-        aby -= af.vgb[j] * b[j];
-        aib += af.bgb[j] * (w[j] - b[j] * bw) + af.vgb[j] * (y[j] - b[j] * by);
+        aw[j] = af.bgb[j] * f.ib;
+        ay[j] = af.vgb[j] * f.ib;
+        ab[j] = af.b[j];
         avE[j] = af.vE[j];
-    }
-    abw *= ib;
-    aby *= ib;
-    // bw = b.w, by = b.y
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        ab[j] += abw * w[j] + aby * y[j];
-        aw[j] += abw * b[j];
-        ay[j] += aby * b[j];
     }
     // w_j = sum_i b_i dB_ij,  y_j = sum_i vE_i dB_ij
 #pragma unroll
-    for (int i = 0; i < ND; ++i)
+    for (int i = 0; i < ND; ++i) {
+        ab[i] += dot3(aw, F.dB[i]);
+        avE[i] += dot3(ay, F.dB[i]);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            ab[i] += aw[j] * F.dB[i][j];
-            avE[i] += ay[j] * F.dB[i][j];
-            aF.dB[i][j] = aw[j] * b[i] + ay[j] * vE[i];
-        }
+        for (int j = 0; j < 3; ++j) aF.dB[i][j] = fma(aw[j], f.b[i], ay[j] * f.vE[i]);
+    }
     // Epar = E.b
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        aF.E[k] = af.Epar * b[k];
-        ab[k] += af.Epar * F.E[k];
-    }
+    for (int k = 0; k < 3; ++k) ab[k] = fma(af.Epar, F.E[k], ab[k]);
     // kappa = (1 - beta2)^(-1/2):  d kappa / d beta2 = kappa^3 / 2
-    const T abeta2 = T(0.5) * af.kappa * kappa * kappa * kappa;
+    const T k2 = af.kappa * f.kappa * f.kappa * f.kappa * inv_c2;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) avE[k] += T(2) * abeta2 * inv_c2 * vE[k];
+    for (int k = 0; k < 3; ++k) avE[k] = fma(k2, f.vE[k], avE[k]);
     // vE = c x ib2,  x = E x B
-    T ax[3], aib2 = T(0);
+    const T cv = c * f.ib2;
+    T ax[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ax[k] = cv * avE[k];
+    const T aib2 = c * dot3(avE, f.x);
+    T tE[3], tB[3];
+    cross3(F.B, ax, tE);
+    cross3(ax, F.E, tB);
+    // b = B ib,  ib2 = ib^2,  ib = 1/|B|,  |B| = sqrt(B.B)
+    aib += dot3(ab, F.B) + T(2) * f.ib * aib2;
+    const T aBmag = af.Bmag - aib * f.ib2;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        ax[k] = c * ib2 * avE[k];
-        aib2 += c * avE[k] * x[k];
+        aF.E[k] = fma(af.Epar, f.b[k], tE[k]);
+        aF.B[k] = fma(ab[k], f.ib, fma(aBmag, f.b[k], tB[k]));
     }
-    T t[3];
-    cross3(F.B, ax, t);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) aF.E[k] += t[k];
-    cross3(ax, F.E, t);
-    // b = B ib,  ib2 = ib^2,  ib = 1/|B|,  |B| = sqrt(B.B)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) aib += ab[k] * F.B[k];
-    aib += T(2) * ib * aib2;
-    const T aBmag = af.Bmag - aib * ib2;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) aF.B[k] = t[k] + ab[k] * ib + aBmag * b[k];
 }
 
-template <typename T>
-__device__ __forceinline__ void perp2_bwd(const Frame<T> &f, const StepPar<T> &s, T mu, T uperp,
-                                          T aP, FrameAdj<T> &af, T &amu, T &auperp)
+template <typename T, typename F>
+__device__ __forceinline__ T perp2_r(const F &f, const StepPar<T> &s, T mu, T uperp)
+{
+    return s.mu_mode ? uperp * uperp : T(2) * mu * f.Bmag * f.kappa;
+}
+template <typename T, typename F>
+__device__ __forceinline__ void perp2_bwd(const F &f, const StepPar<T> &s, T mu, T uperp, T aP,
+                                          FrameAdj<T> &af, T &amu, T &auperp)
 {
     if (s.mu_mode) {
-        auperp += T(2) * uperp * aP;
+        auperp = fma(T(2) * uperp, aP, auperp);
     } else {
-        amu += T(2) * f.Bmag * f.kappa * aP;
-        af.Bmag += T(2) * mu * f.kappa * aP;
-        af.kappa += T(2) * mu * f.Bmag * aP;
+        const T a2 = T(2) * aP;
+        amu = fma(f.Bmag * f.kappa, a2, amu);
+        af.Bmag = fma(mu * f.kappa, a2, af.Bmag);
+        af.kappa = fma(mu * f.Bmag, a2, af.kappa);
     }
 }
 
-// Gamma = kappa sqrt(1 + (u_par^2 + P)/c^2)
+// Gamma = kappa S, S = sqrt(1 + (u_par^2 + P)/c^2), with its reciprocals
 template <typename T>
-__device__ __forceinline__ void gamma_gc_bwd(const Frame<T> &f, const StepPar<T> &s, T upar,
-                                             T mu, T uperp, T aG, FrameAdj<T> &af, T &aupar,
-                                             T &amu, T &auperp)
+struct Gam { T S, iS, G, iG; };
+
+template <typename T, typename F>
+__device__ __forceinline__ Gam<T> gamma_r(const F &f, const StepPar<T> &s, T upar, T mu, T uperp)
 {
-    const T P = perp2(f, s, mu, uperp);
-    const T S = sqrt(T(1) + fma(upar, upar, P) * s.inv_c2);
-    af.kappa += aG * S;
-    const T ain = aG * f.kappa * s.inv_c2 / (T(2) * S);
-    aupar += T(2) * upar * ain;
+    Gam<T> g;
+    const T S2 = fma(fma(upar, upar, perp2_r(f, s, mu, uperp)), s.inv_c2, T(1));
+    g.iS = rsq_r(S2);
+    g.S = S2 * g.iS;
+    g.G = f.kappa * g.S;
+    g.iG = f.ikap * g.iS;
+    return g;
+}
+template <typename T, typename F>
+__device__ __forceinline__ void gamma_bwd(const F &f, const StepPar<T> &s, const Gam<T> &g, T upar,
+                                          T mu, T uperp, T aG, FrameAdj<T> &af, T &aupar, T &amu,
+                                          T &auperp)
+{
+    af.kappa = fma(aG, g.S, af.kappa);
+    const T ain = T(0.5) * aG * f.kappa * s.inv_c2 * g.iS;
+    aupar = fma(T(2) * upar, ain, aupar);
     perp2_bwd(f, s, mu, uperp, ain, af, amu, auperp);
 }
 
 // v_c = pref b x (k2 bgb + u_par vgb),  k2 = u_par^2/G,  pref = c kappa^2/(q/m |B|)
-template <typename T>
-__device__ __forceinline__ void vcurv_bwd(const Frame<T> &f, const StepPar<T> &s, T upar, T G,
+template <typename T, typename F>
+__device__ __forceinline__ void vcurv_r(const F &f, const StepPar<T> &s, T upar, T iG, T vc[3])
+{
+    if (!s.curvature) { vc[0] = vc[1] = vc[2] = T(0); return; }
+    T a[3], x[3];
+    const T k2 = upar * upar * iG;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) a[k] = fma(k2, f.bgb[k], upar * f.vgb[k]);
+    cross3(f.b, a, x);
+    const T pref = s.cq * f.kappa * f.kappa * f.ib;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) vc[k] = pref * x[k];
+}
+template <typename T, typename F>
+__device__ __forceinline__ void vcurv_bwd(const F &f, const StepPar<T> &s, T upar, T iG,
                                           const T avc[3], FrameAdj<T> &af, T &aupar, T &aG)
 {
     if (!s.curvature) return;
-    const T k2 = upar * upar / G;
+    const T ig = upar * iG, k2 = upar * ig;
     T a[3], x[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) a[k] = fma(k2, f.bgb[k], upar * f.vgb[k]);
     cross3(f.b, a, x);
-    const T pref = s.c * f.kappa * f.kappa / (s.qm * f.Bmag);
-    const T apref = dot3(avc, x);
+    const T pref = s.cq * f.kappa * f.kappa * f.ib;
+    const T apref = pref * dot3(avc, x);
     T ax[3], t[3], aa[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) ax[k] = pref * avc[k];
@@ -168,35 +200,34 @@ __device__ __forceinline__ void vcurv_bwd(const Frame<T> &f, const StepPar<T> &s
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         af.b[k] += t[k];
-        af.bgb[k] += k2 * aa[k];
-        af.vgb[k] += upar * aa[k];
+        af.bgb[k] = fma(k2, aa[k], af.bgb[k]);
+        af.vgb[k] = fma(upar, aa[k], af.vgb[k]);
     }
     const T ak2 = dot3(aa, f.bgb);
-    aupar += dot3(aa, f.vgb) + T(2) * upar / G * ak2;
-    aG -= k2 / G * ak2;
-    af.kappa += T(2) * pref / f.kappa * apref;
-    af.Bmag -= pref / f.Bmag * apref;
+    aupar += fma(T(2) * ig, ak2, dot3(aa, f.vgb));
+    aG = fma(-ig * ig, ak2, aG);
+    af.kappa = fma(T(2) * f.ikap, apref, af.kappa);
+    af.Bmag = fma(-f.ib, apref, af.Bmag);
 }
 
 // V = (u_par/G) b + vE + v_c,  G = Gamma(u_par, mu)
-template <typename T>
-__device__ __forceinline__ void gc_vel_bwd(const Frame<T> &f, const StepPar<T> &s, T upar, T mu,
-                                           T uperp, const T aV[3], FrameAdj<T> &af, T &aupar,
-                                           T &amu, T &auperp)
+template <typename T, typename F>
+__device__ __forceinline__ void gc_vel_bwd(const F &f, const StepPar<T> &s, T upar, T mu, T uperp,
+                                           const T aV[3], FrameAdj<T> &af, T &aupar, T &amu,
+                                           T &auperp)
 {
-    const T G = gamma_gc(f, s, upar, mu, uperp);
-    const T ig = upar / G;
-    const T aig = dot3(aV, f.b);
+    const Gam<T> g = gamma_r(f, s, upar, mu, uperp);
+    const T ig = upar * g.iG;
+    const T aig = dot3(aV, f.b) * g.iG;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        af.b[k] += ig * aV[k];
+        af.b[k] = fma(ig, aV[k], af.b[k]);
         af.vE[k] += aV[k];
     }
-    T aG = T(0);
-    vcurv_bwd(f, s, upar, G, aV, af, aupar, aG);
-    aupar += aig / G;
-    aG -= ig / G * aig;
-    gamma_gc_bwd(f, s, upar, mu, uperp, aG, af, aupar, amu, auperp);
+    aupar += aig;
+    T aG = -ig * aig;
+    vcurv_bwd(f, s, upar, g.iG, aV, af, aupar, aG);
+    gamma_bwd(f, s, g, upar, mu, uperp, aG, af, aupar, amu, auperp);
 }
 
 // u_par update at x^n (Sec. 2.2.1 without curvature; Sec. 2.2.2 with it: the
@@ -204,70 +235,87 @@ __device__ __forceinline__ void gc_vel_bwd(const Frame<T> &f, const StepPar<T> &
 // derivative follows from the quadratic itself: dG1 = -(G1^2 dk1 + G1 dk2 +
 // dk3) / (2 k1 G1 + k2)).
 template <typename T>
-__device__ __forceinline__ void upar_bwd(const Frame<T> &f0, const StepPar<T> &s, T upar, T mu,
-                                         T uperp, T aupn, FrameAdj<T> &af, T &aupar, T &amu,
-                                         T &auperp)
+struct Quad { T A, gg, D, iD, upr, P0, k1, k2, G1, upn; Gam<T> g0; };
+
+// (rG: the root chosen as the forward step does, the larger of the two)
+template <typename T, typename F>
+__device__ __forceinline__ void quad_r(const F &f0, const StepPar<T> &s, T upar, T mu, T uperp, Quad<T> &q)
+{
+    q.A = dot3(f0.vE, f0.bgb);
+    q.gg = dot3(f0.vE, f0.vgb);
+    q.D = fma(-s.half_dt, q.A, T(1));
+    q.iD = rcp_r(q.D);
+    q.g0 = gamma_r(f0, s, upar, mu, uperp);
+    q.upr = fma(upar, fma(s.half_dt, q.A, T(1)),
+                fma(s.qm * s.dt, f0.Epar, s.half_dt * q.g0.G * q.gg));
+    const T c2 = s.c * s.c, D2 = q.D * q.D;
+    q.P0 = perp2_r(f0, s, mu, uperp);
+    q.k1 = T(0.25) * s.dt * s.dt * q.gg * q.gg - c2 * D2 * f0.om;
+    q.k2 = q.upr * s.dt * q.gg;
+    const T k3 = fma(q.upr, q.upr, (c2 + q.P0) * D2);
+    const T disc = fma(q.k2, q.k2, T(-4) * q.k1 * k3);
+    const T sq = disc * rsq_r(disc);
+    const T h = T(-0.5) * (q.k2 + (q.k2 >= T(0) ? sq : -sq));
+    q.G1 = q.k2 >= T(0) ? h * rcp_r(q.k1) : k3 * rcp_r(h);
+    q.upn = fma(s.half_dt * q.G1, q.gg, q.upr) * q.iD;
+}
+
+// u_par^{n+1/2} from the frame at x^n
+template <typename T, typename F>
+__device__ __forceinline__ T upar_new(const F &f0, const StepPar<T> &s, T upar, T mu, T uperp)
+{
+    if (!s.curvature) return fma(s.qm * s.dt, f0.Epar, upar);
+    Quad<T> q;
+    quad_r(f0, s, upar, mu, uperp, q);
+    return q.upn;
+}
+
+template <typename T, typename F>
+__device__ __forceinline__ void upar_bwd(const F &f0, const StepPar<T> &s, T upar, T mu, T uperp,
+                                         T aupn, FrameAdj<T> &af, T &aupar, T &amu, T &auperp)
 {
     if (!s.curvature) {
         aupar += aupn;
-        af.Epar += s.qm * s.dt * aupn;
+        af.Epar = fma(s.qm * s.dt, aupn, af.Epar);
         return;
     }
-    const T A = dot3(f0.vE, f0.bgb);
-    const T gg = dot3(f0.vE, f0.vgb);
-    const T D = fma(-s.half_dt, A, T(1));
-    const T G0 = gamma_gc(f0, s, upar, mu, uperp);
-    const T upr = fma(upar, fma(s.half_dt, A, T(1)), fma(s.qm * s.dt, f0.Epar, s.half_dt * G0 * gg));
+    Quad<T> q;
+    quad_r(f0, s, upar, mu, uperp, q);
     const T c2 = s.c * s.c;
-    const T kap2 = f0.kappa * f0.kappa;
-    const T P0 = perp2(f0, s, mu, uperp);
-    const T k1 = T(0.25) * s.dt * s.dt * gg * gg - c2 * D * D / kap2;
-    const T k2 = upr * s.dt * gg;
-    const T k3 = fma(upr, upr, (c2 + P0) * D * D);
-    const T disc = fma(k2, k2, T(-4) * k1 * k3);
-    const T sq = sqrt(disc);
-    const T q = T(-0.5) * (k2 + (k2 >= T(0) ? sq : -sq));
-    const T r1 = q / k1;
-    const T r2 = (q != T(0)) ? k3 / q : T(-1);
-    const T G1 = r1 >= r2 ? r1 : r2;
-    const T upn = fma(s.half_dt * G1, gg, upr) / D;
-
-    const T iD = T(1) / D;
-    const T aG1 = aupn * s.half_dt * gg * iD;
-    T agg = aupn * s.half_dt * G1 * iD;
-    T aupr = aupn * iD;
-    T aD = -aupn * upn * iD;
-    const T den = fma(T(2) * k1, G1, k2);
-    const T ak1 = -aG1 * G1 * G1 / den;
-    const T ak2 = -aG1 * G1 / den;
-    const T ak3 = -aG1 / den;
+    const T av = aupn * q.iD;
+    const T aG1 = av * s.half_dt * q.gg;
+    T agg = av * s.half_dt * q.G1;
+    T aupr = av;
+    T aD = -av * q.upn;
+    const T ak3 = -aG1 * rcp_r(fma(T(2) * q.k1, q.G1, q.k2));
+    const T ak2 = q.G1 * ak3;
+    const T ak1 = q.G1 * ak2;
     // k3 = upr^2 + (c^2 + P0) D^2
-    aupr += T(2) * upr * ak3;
-    const T aP0 = D * D * ak3;
-    aD += T(2) * (c2 + P0) * D * ak3;
+    aupr = fma(T(2) * q.upr, ak3, aupr);
+    const T aP0 = q.D * q.D * ak3;
+    aD = fma(T(2) * (c2 + q.P0) * q.D, ak3, aD);
     // k2 = upr dt gg
-    aupr += s.dt * gg * ak2;
-    agg += upr * s.dt * ak2;
+    aupr = fma(s.dt * q.gg, ak2, aupr);
+    agg = fma(q.upr * s.dt, ak2, agg);
     // k1 = dt^2 gg^2 / 4 - c^2 D^2 / kappa^2
-    agg += T(0.5) * s.dt * s.dt * gg * ak1;
-    aD -= T(2) * c2 * D / kap2 * ak1;
-    af.kappa += T(2) * c2 * D * D / (kap2 * f0.kappa) * ak1;
+    agg = fma(T(0.5) * s.dt * s.dt * q.gg, ak1, agg);
+    aD = fma(T(-2) * c2 * q.D * f0.om, ak1, aD);
+    af.kappa = fma(T(2) * c2 * q.D * q.D * f0.om * f0.ikap, ak1, af.kappa);
     // upr = u_par (1 + dt/2 A) + (q/m) dt Epar + dt/2 G0 gg
-    aupar += fma(s.half_dt, A, T(1)) * aupr;
-    T aA = upar * s.half_dt * aupr;
-    af.Epar += s.qm * s.dt * aupr;
-    const T aG0 = s.half_dt * gg * aupr;
-    agg += s.half_dt * G0 * aupr;
+    aupar = fma(fma(s.half_dt, q.A, T(1)), aupr, aupar);
     // D = 1 - dt/2 A
-    aA -= s.half_dt * aD;
-    gamma_gc_bwd(f0, s, upar, mu, uperp, aG0, af, aupar, amu, auperp);
+    const T aA = s.half_dt * fma(upar, aupr, -aD);
+    af.Epar = fma(s.qm * s.dt, aupr, af.Epar);
+    const T aG0 = s.half_dt * q.gg * aupr;
+    agg = fma(s.half_dt * q.g0.G, aupr, agg);
+    gamma_bwd(f0, s, q.g0, upar, mu, uperp, aG0, af, aupar, amu, auperp);
     perp2_bwd(f0, s, mu, uperp, aP0, af, amu, auperp);
     // gg = vE.vgb,  A = vE.bgb
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        af.vE[k] += agg * f0.vgb[k] + aA * f0.bgb[k];
-        af.vgb[k] += agg * f0.vE[k];
-        af.bgb[k] += aA * f0.vE[k];
+        af.vE[k] += fma(agg, f0.vgb[k], aA * f0.bgb[k]);
+        af.vgb[k] = fma(agg, f0.vE[k], af.vgb[k]);
+        af.bgb[k] = fma(aA, f0.vE[k], af.bgb[k]);
     }
 }
 
@@ -275,96 +323,103 @@ __device__ __forceinline__ void upar_bwd(const Frame<T> &f0, const StepPar<T> &s
 // u_g = u - u_par b - (vE + v_c(u_par, G)) G,  u_perp = |u_g|, bpg = u_g/u_perp,
 // mu = u_perp^2 / (2 |B| kappa).
 template <typename T>
-__device__ __forceinline__ void conv_fwd(const Frame<T> &fm, const StepPar<T> &s, const T u[3],
-                                         T &Gf, T &upar, T vc[3], T &uperp, T &mu, T bpg[3])
+struct Conv { T G, iG, upar, vc[3], uperp, iu, mu, bpg[3]; };
+
+template <typename T, typename F>
+__device__ __forceinline__ void conv_fwd(const F &fm, const StepPar<T> &s, const T u[3], Conv<T> &q)
 {
-    Gf = sqrt(T(1) + dot3(u, u) * s.inv_c2);
-    upar = dot3(u, fm.b);
-    vcurv(fm, s, upar, Gf, vc);
+    const T G2 = fma(dot3(u, u), s.inv_c2, T(1));
+    q.iG = rsq_r(G2);
+    q.G = G2 * q.iG;
+    q.upar = dot3(u, fm.b);
+    vcurv_r(fm, s, q.upar, q.iG, q.vc);
     T ug[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) ug[k] = u[k] - upar * fm.b[k] - (fm.vE[k] + vc[k]) * Gf;
-    uperp = sqrt(dot3(ug, ug));
-    if (uperp < Eps<T>::tiny) {
-        uperp = T(0);
-        mu = T(0);
-        bpg[0] = bpg[1] = bpg[2] = T(0);
+    for (int k = 0; k < 3; ++k) ug[k] = fma(-q.G, fm.vE[k] + q.vc[k], fma(-q.upar, fm.b[k], u[k]));
+    const T up2 = dot3(ug, ug);
+    q.iu = rsq_r(up2);
+    q.uperp = up2 * q.iu;
+    if (!(q.uperp >= Eps<T>::tiny)) {
+        q.uperp = q.iu = q.mu = T(0);
+        q.bpg[0] = q.bpg[1] = q.bpg[2] = T(0);
     } else {
-        const T iu = T(1) / uperp;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) bpg[k] = ug[k] * iu;
-        mu = uperp * uperp / (T(2) * fm.Bmag * fm.kappa);
+        for (int k = 0; k < 3; ++k) q.bpg[k] = ug[k] * q.iu;
+        q.mu = T(0.5) * up2 * fm.ib * fm.ikap;
     }
 }
 
-template <typename T>
-__device__ __forceinline__ void conv_bwd(const Frame<T> &fm, const StepPar<T> &s, const T u[3],
-                                         T Gf, T upar, const T vc[3], T uperp, T mu,
-                                         const T bpg[3], T aupar, T amu, T auperp,
-                                         const T abpg[3], FrameAdj<T> &af, T au[3])
+template <typename T, typename F>
+__device__ __forceinline__ void conv_bwd(const F &fm, const StepPar<T> &s, const T u[3],
+                                         const Conv<T> &q, T aupar, T amu, T auperp, const T abpg[3],
+                                         FrameAdj<T> &af, T au[3])
 {
     T aug[3] = {T(0), T(0), T(0)};
-    if (uperp > T(0)) {
-        auperp += amu * uperp / (fm.Bmag * fm.kappa);
-        af.Bmag -= amu * mu / fm.Bmag;
-        af.kappa -= amu * mu / fm.kappa;
-        const T abb = dot3(abpg, bpg);
-        const T iu = T(1) / uperp;
+    if (q.uperp > T(0)) {
+        auperp = fma(amu * q.uperp, fm.ib * fm.ikap, auperp);
+        af.Bmag = fma(-amu * q.mu, fm.ib, af.Bmag);
+        af.kappa = fma(-amu * q.mu, fm.ikap, af.kappa);
+        const T abb = dot3(abpg, q.bpg);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) aug[k] = (abpg[k] - abb * bpg[k]) * iu + auperp * bpg[k];
+        for (int k = 0; k < 3; ++k)
+            aug[k] = fma(fma(-abb, q.bpg[k], abpg[k]), q.iu, auperp * q.bpg[k]);
     }
     T avc[3];
     T aGf = T(0);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         au[k] += aug[k];
-        af.b[k] -= upar * aug[k];
-        af.vE[k] -= Gf * aug[k];
-        avc[k] = -Gf * aug[k];
-        aGf -= aug[k] * (fm.vE[k] + vc[k]);
+        af.b[k] = fma(-q.upar, aug[k], af.b[k]);
+        af.vE[k] = fma(-q.G, aug[k], af.vE[k]);
+        avc[k] = -q.G * aug[k];
+        aGf = fma(-aug[k], fm.vE[k] + q.vc[k], aGf);
     }
     aupar -= dot3(aug, fm.b);
-    vcurv_bwd(fm, s, upar, Gf, avc, af, aupar, aGf);
+    vcurv_bwd(fm, s, q.upar, q.iG, avc, af, aupar, aGf);
+    const T ag = aGf * s.inv_c2 * q.iG;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        au[k] += aupar * fm.b[k] + aGf * u[k] * s.inv_c2 / Gf;
-        af.b[k] += aupar * u[k];
+        au[k] += fma(aupar, fm.b[k], ag * u[k]);
+        af.b[k] = fma(aupar, u[k], af.b[k]);
     }
 }
 
 // Reconstruction at R^{n+1/2}:  u = u_par b + (vE + v_c) G + u_n bpg,
 // u_n = u_perp (mu_mode) or sqrt(2 mu |B| kappa).
-template <typename T>
-__device__ __forceinline__ void recon_bwd(const Frame<T> &fp, const StepPar<T> &s, T upn, T mu,
-                                          T uperp, const T bpg[3], const T lamu[3],
-                                          FrameAdj<T> &af, T &aupn, T &amu, T &auperp, T abpg[3])
+template <typename T, typename F>
+__device__ __forceinline__ void recon_bwd(const F &fp, const StepPar<T> &s, T upn, T mu, T uperp,
+                                          const T bpg[3], const T lamu[3], FrameAdj<T> &af, T &aupn,
+                                          T &amu, T &auperp, T abpg[3])
 {
-    const T Gp = gamma_gc(fp, s, upn, mu, uperp);
+    const Gam<T> g = gamma_r(fp, s, upn, mu, uperp);
     T vc[3];
-    vcurv(fp, s, upn, Gp, vc);
-    const T un = s.mu_mode ? uperp : sqrt(T(2) * mu * fp.Bmag * fp.kappa);
+    vcurv_r(fp, s, upn, g.iG, vc);
+    const T Bk = fp.Bmag * fp.kappa;
+    const T un2 = T(2) * mu * Bk;
+    const T iun = un2 > T(0) ? rsq_r(un2) : T(0);
+    const T un = s.mu_mode ? uperp : un2 * iun;
     aupn += dot3(lamu, fp.b);
     T avc[3];
     T aGp = T(0);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        af.b[k] += upn * lamu[k];
-        af.vE[k] += Gp * lamu[k];
-        abpg[k] += un * lamu[k];
-        avc[k] = Gp * lamu[k];
-        aGp += lamu[k] * (fp.vE[k] + vc[k]);
+        af.b[k] = fma(upn, lamu[k], af.b[k]);
+        af.vE[k] = fma(g.G, lamu[k], af.vE[k]);
+        abpg[k] = fma(un, lamu[k], abpg[k]);
+        avc[k] = g.G * lamu[k];
+        aGp = fma(lamu[k], fp.vE[k] + vc[k], aGp);
     }
     const T aun = dot3(lamu, bpg);
     if (s.mu_mode) {
         auperp += aun;
-    } else if (un > T(0)) {
-        const T iun = T(1) / un;
-        amu += aun * fp.Bmag * fp.kappa * iun;
-        af.Bmag += aun * mu * fp.kappa * iun;
-        af.kappa += aun * mu * fp.Bmag * iun;
+    } else {
+        const T t = aun * iun;
+        amu = fma(t, Bk, amu);
+        af.Bmag = fma(t * mu, fp.kappa, af.Bmag);
+        af.kappa = fma(t * mu, fp.Bmag, af.kappa);
     }
-    vcurv_bwd(fp, s, upn, Gp, avc, af, aupn, aGp);
-    gamma_gc_bwd(fp, s, upn, mu, uperp, aGp, af, aupn, amu, auperp);
+    vcurv_bwd(fp, s, upn, g.iG, avc, af, aupn, aGp);
+    gamma_bwd(fp, s, g, upn, mu, uperp, aGp, af, aupn, amu, auperp);
 }
 
 // Relativistic Boris push (Sec. 2.1) and disp = dt u/gamma: adjoints of u, E, B.

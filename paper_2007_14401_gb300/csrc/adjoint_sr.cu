@@ -23,40 +23,12 @@
 #include "gca_lean.cuh"
 #include "push_sr.cuh"
 
-// Code size of the reverse kernel: its per-point pieces (gather + frame,
-// frame transpose + scatter, and at level 2 the guiding-center velocity
-// transpose and the replay's gather) are called out of line instead of being
-// inlined at every gather point, which keeps the kernel's instruction
-// footprint within the instruction caches.
-#ifndef GCB_ADJ_OUTLINE
-#define GCB_ADJ_OUTLINE 0
-#endif
-// GCB_ADJ_CACHE: cells (0, 1 or 2) whose node adjoints a thread accumulates
-// in shared memory over a particle-step before adding them to the FP64 node
-// accumulators (0: every gather's contributions are added directly).
-#ifndef GCB_ADJ_CACHE
-#define GCB_ADJ_CACHE 1
-#endif
 // GCB_ADJ_FCACHE: gather points (x^n first, then the step's gathers in order)
 // whose interpolated field the replay keeps in shared memory for the reverse
 // loop, which otherwise gathers again; points past it are re-gathered.
 #ifndef GCB_ADJ_FCACHE
 #define GCB_ADJ_FCACHE 6
 #endif
-#ifndef GCB_ADJ_BLOCKS_F32
-#define GCB_ADJ_BLOCKS_F32 4
-#endif
-#if GCB_ADJ_OUTLINE >= 1
-#define GCB_ADJ_FN1 __device__ __noinline__
-#else
-#define GCB_ADJ_FN1 __device__ __forceinline__
-#endif
-#if GCB_ADJ_OUTLINE >= 2
-#define GCB_ADJ_FN2 __device__ __noinline__
-#else
-#define GCB_ADJ_FN2 __device__ __forceinline__
-#endif
-
 namespace gcb {
 namespace adj {
 
@@ -299,38 +271,79 @@ __global__ void __launch_bounds__(TPB) k_adjoint_sr(const AdjArgs<T> a)
 // transposed step backwards (adjoint_rev.cuh), re-gathering at each point.
 // ---------------------------------------------------------------------------
 
+// Per-thread values in shared memory, 16 bytes at a time: chunk j of the
+// block's thread t at [j * TPB + t], so that a quarter warp's accesses fill the
+// banks and 12 components are 3 (FP64: 6) loads or stores instead of 12.
 template <typename T>
-GCB_ADJ_FN2 void plain_gather2(const DevGrid<T> &g, const int ib[2], const T l[2], FieldPt<T, 2> &F)
+struct alignas(16) Vec {
+    static constexpr int n = Chunk<T>::n;
+    T v[n];
+};
+template <typename T>
+constexpr int kChunks = NF / Chunk<T>::n;      // chunks of one point's 12 components
+
+__device__ __forceinline__ void axpy(float W, const Vec<float> &x, Vec<float> &y)
 {
-    gather<T, 2, 2>(g, ib, l, F);
+    const float2 w = make_float2(W, W);
+    const float2 a = __ffma2_rn(make_float2(x.v[0], x.v[1]), w, make_float2(y.v[0], y.v[1]));
+    const float2 b = __ffma2_rn(make_float2(x.v[2], x.v[3]), w, make_float2(y.v[2], y.v[3]));
+    y.v[0] = a.x; y.v[1] = a.y; y.v[2] = b.x; y.v[3] = b.y;
+}
+__device__ __forceinline__ void axpy(double W, const Vec<double> &x, Vec<double> &y)
+{
+    y.v[0] = fma(W, x.v[0], y.v[0]);
+    y.v[1] = fma(W, x.v[1], y.v[1]);
+}
+
+// a field point as 16-byte chunks: E, B, d_x B, d_y B
+template <typename T>
+__device__ __forceinline__ void to_chunks(const FieldPt<T, 2> &F, Vec<T> q[kChunks<T>])
+{
+    T v[NF];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        v[c] = F.E[c];
+        v[3 + c] = F.B[c];
+        v[6 + c] = F.dB[0][c];
+        v[9 + c] = F.dB[1][c];
+    }
+#pragma unroll
+    for (int c = 0; c < NF; ++c) q[c / Vec<T>::n].v[c % Vec<T>::n] = v[c];
+}
+template <typename T>
+__device__ __forceinline__ void from_chunks(const Vec<T> q[kChunks<T>], FieldPt<T, 2> &F)
+{
+    T v[NF];
+#pragma unroll
+    for (int c = 0; c < NF; ++c) v[c] = q[c / Vec<T>::n].v[c % Vec<T>::n];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        F.E[c] = v[c];
+        F.B[c] = v[3 + c];
+        F.dB[0][c] = v[6 + c];
+        F.dB[1][c] = v[9 + c];
+    }
 }
 
 // Interpolated fields of the step's gather points, kept per thread in shared
-// memory (thread-fastest: element (point, component) at [(point*NF+c)*TPB]).
-// Point 0 is x^n, point 1 + k the step's k-th gather.
+// memory.  Point 0 is x^n, point 1 + k the step's k-th gather.
 template <typename T>
 struct FCache {
-    T *base;
+    Vec<T> *base;
     __device__ __forceinline__ void store(int pt, const FieldPt<T, 2> &F) const
     {
         if (pt >= GCB_ADJ_FCACHE) return;
-        T *q = base + pt * NF * TPB;
+        Vec<T> q[kChunks<T>];
+        to_chunks(F, q);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) { q[c * TPB] = F.E[c]; q[(3 + c) * TPB] = F.B[c]; }
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) q[(6 + 3 * i + j) * TPB] = F.dB[i][j];
+        for (int j = 0; j < kChunks<T>; ++j) base[(pt * kChunks<T> + j) * TPB] = q[j];
     }
     __device__ __forceinline__ void load(int pt, FieldPt<T, 2> &F) const
     {
-        const T *q = base + pt * NF * TPB;
+        Vec<T> q[kChunks<T>];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) { F.E[c] = q[c * TPB]; F.B[c] = q[(3 + c) * TPB]; }
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) F.dB[i][j] = q[(6 + 3 * i + j) * TPB];
+        for (int j = 0; j < kChunks<T>; ++j) q[j] = base[(pt * kChunks<T> + j) * TPB];
+        from_chunks(q, F);
     }
 };
 
@@ -349,182 +362,180 @@ struct RecGather {
             pts[k][0] = l[0];
             pts[k][1] = l[1];
         }
-        plain_gather2(g, ib, l, F);
+        gather_any<T, 2, 2>(g, ib, l, F);
         fc.store(1 + k, F);
     }
 };
 
-// Node-record adjoints of one particle-step, accumulated per thread for up
-// to GCB_ADJ_CACHE cells (4 nodes x 12 components each) in shared memory laid
-// out thread-fastest, and added to the FP64 node accumulators when a cell is
-// evicted and at the end of the step: the step's gathers (x^n, R^{n-1/2},
-// the iterates, R^{n+1/2}) mostly share one cell, so this replaces most of
-// the per-gather atomics.  (One cell measured faster than two: the second
-// costs shared memory that the field cache uses better.)
+// Node-record adjoints of one particle-step, accumulated per thread for one
+// cell (4 nodes x 12 components) in shared memory and added to the FP64 node
+// accumulators when the cell changes and at the end of the step: the step's
+// gathers (x^n, R^{n-1/2}, the iterates, R^{n+1/2}) mostly share one cell, so
+// this replaces most of the per-gather atomics.  (One cell measured faster
+// than two: the second costs shared memory that the field cache uses better.)
+// The additions are made by the warp together, two threads' cells at a time,
+// 16 lanes each: a lane's 48 additions on its own go to 48 separate sectors
+// one by one, here 16 lanes add to 128 contiguous bytes.  The chunks of a
+// thread are (TPB + 1) apart, which puts the 16 values read together in 16
+// different banks.
 template <typename T>
 struct NodeCache {
-    T *acc;          // this thread's slot 0 element; element (s, o, c) at acc[((s*4+o)*NF+c)*TPB]
+    static constexpr int LD = TPB + 1;
+    static constexpr int N = 4 * kChunks<T> * LD;   // chunks of a block
+    Vec<T> *base;    // chunk (o, j) of the block's thread t at base[(o * kChunks + j) * LD + t]
     double *grad;
     int nx, ny;
-    int key[2];      // lower-left node of the cached cell, -1 when empty
-    int mru;         // most recently used slot
+    int cx, cy;      // the cached cell, cx = -1 when empty
 
-    __device__ __forceinline__ T &at(int sl, int o, int c) const
+    __device__ __forceinline__ Vec<T> &at(int o, int j) const
     {
-        return acc[((sl * 4 + o) * NF + c) * TPB];
+        return base[(o * kChunks<T> + j) * LD + threadIdx.x];
     }
-    __device__ __forceinline__ void flush(int sl)
+    // add the cached cells of the lanes that ask for it (called by the whole warp)
+    __device__ __forceinline__ void flush(bool want)
     {
-        const int k = sl ? key[1] : key[0];
-        if (k < 0) return;
-        const int ix = k % nx, iy = k / nx;
-        const int jx = ix + 1 == nx ? 0 : ix + 1, jy = iy + 1 == ny ? 0 : iy + 1;
+        unsigned m = __ballot_sync(0xffffffffu, want && cx >= 0);
+        const int lane = threadIdx.x & 31, h = lane & 15;
+        __syncwarp();
+        while (m) {
+            const int a = __ffs(m) - 1;
+            m &= m - 1;
+            const int b = m ? __ffs(m) - 1 : a;
+            const bool act = lane < 16 || m;
+            m &= m - 1;
+            const int src = lane < 16 ? a : b;
+            const int ix = __shfl_sync(0xffffffffu, cx, src), iy = __shfl_sync(0xffffffffu, cy, src);
+            const int jx = ix + 1 == nx ? 0 : ix + 1, jy = iy + 1 == ny ? 0 : iy + 1;
+            const T *v = reinterpret_cast<const T *>(base + (threadIdx.x & ~31) + src);
 #pragma unroll
-        for (int o = 0; o < 4; ++o) {
-            const int node = ((o & 2) ? jy : iy) * nx + ((o & 1) ? jx : ix);
-            double *gp = grad + (size_t)node * NF;
-#pragma unroll
-            for (int c = 0; c < NF; ++c) {
-                const T v = at(sl, o, c);
-                if (v != T(0)) atomicAdd(gp + c, (double)v);
+            for (int k = 0; k < 3; ++k) {
+                const int e = h + 16 * k, o = e / NF, c = e - o * NF;   // node and component
+                const T x = v[(e / Vec<T>::n) * (LD * Vec<T>::n) + e % Vec<T>::n];
+                const int node = ((o & 2) ? jy : iy) * nx + ((o & 1) ? jx : ix);
+                if (act && x != T(0)) atomicAdd(grad + (size_t)node * NF + c, (double)x);
             }
         }
+        __syncwarp();
     }
-    // slot holding cell `k` (evicting the least recently used one if needed)
-    __device__ __forceinline__ int slot(int k)
+    // make cell (ix, iy) the cached one of the lanes in `on` (called by the whole warp)
+    __device__ __forceinline__ void select(bool on, int ix, int iy)
     {
-        int sl;
-        if (k == key[0]) {
-            sl = 0;
-        } else if (GCB_ADJ_CACHE > 1 && k == key[1]) {
-            sl = 1;
-        } else {
-            sl = GCB_ADJ_CACHE > 1 ? 1 - mru : 0;
-            flush(sl);
-            if (sl) key[1] = k; else key[0] = k;
+        const bool other = on && (ix != cx || iy != cy);
+        flush(other);
+        if (!other) return;
+        cx = ix;
+        cy = iy;
+        Vec<T> z;
 #pragma unroll
-            for (int o = 0; o < 4; ++o)
+        for (int c = 0; c < Vec<T>::n; ++c) z.v[c] = T(0);
 #pragma unroll
-                for (int c = 0; c < NF; ++c) at(sl, o, c) = T(0);
-        }
-        mru = sl;
-        return sl;
+        for (int o = 0; o < 4; ++o)
+#pragma unroll
+            for (int j = 0; j < kChunks<T>; ++j) at(o, j) = z;
     }
     __device__ __forceinline__ void finish()
     {
-        flush(0);
-        if (GCB_ADJ_CACHE > 1) flush(1);
-        key[0] = key[1] = -1;
+        flush(true);
+        cx = -1;
     }
 };
 
-// Transpose of F = sum_o W_o(p) rec_o: the node records receive W_o aF (via
-// the cache) and the position adjoint sum_o grad W_o (rec_o . aF) is returned.
+// Cell of a gather point: fractional position, cell and the nodes' record
+// indices (both ways of finding them as the gather's own).
 template <typename T>
-__device__ __forceinline__ void gather_bwd(const DevGrid<T> &g, NodeCache<T> &nc, const int ib[2],
-                                           const T p[2], const FieldPt<T, 2> &aF, T ap[2])
+__device__ __forceinline__ void cell_nodes(const DevGrid<T> &g, const int ib[2], const T p[2], T t[2],
+                                           int i0[2], int node[4])
 {
-    int i0[2], i1[2];
-    T t[2];
+    int i1[2];
 #pragma unroll
     for (int d = 0; d < 2; ++d) cell_of(g, d, ib[d], p[d], t[d], i0[d], i1[d]);
-    T av[NF];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) { av[c] = aF.E[c]; av[3 + c] = aF.B[c]; }
+    for (int o = 0; o < 4; ++o)
+        node[o] = ((o & 2) ? i1[1] : i0[1]) * g.n[0] + ((o & 1) ? i1[0] : i0[0]);
+}
+template <>
+__device__ __forceinline__ void cell_nodes<float>(const DevGrid<float> &g, const int ib[2],
+                                                  const float p[2], float t[2], int i0[2],
+                                                  int node[4])
+{
+    CellLoc<2> q;
+    locate<2>(g, ib, p, q);
+    t[0] = q.t[0];
+    t[1] = q.t[1];
+    if (q.inner) {
+        i0[0] = q.i[0];
+        i0[1] = q.i[1];
+        node[0] = q.i[1] * g.n[0] + q.i[0];
+        node[1] = node[0] + 1;
+        node[2] = node[0] + g.n[0];
+        node[3] = node[2] + 1;
+    } else {
+        int i1[2];
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) av[6 + 3 * i + j] = aF.dB[i][j];
-#if GCB_ADJ_CACHE
-    const int sl = nc.slot(i0[1] * g.n[0] + i0[0]);
-#endif
-    ap[0] = ap[1] = T(0);
-#pragma unroll
-    for (int o = 0; o < 4; ++o) {
-        const int ix = (o & 1) ? i1[0] : i0[0];
-        const int iy = (o & 2) ? i1[1] : i0[1];
-        const int node = iy * g.n[0] + ix;
-        const T wx = (o & 1) ? t[0] : T(1) - t[0];
-        const T wy = (o & 2) ? t[1] : T(1) - t[1];
-        const T dwx = (o & 1) ? g.inv_dx[0] : -g.inv_dx[0];
-        const T dwy = (o & 2) ? g.inv_dx[1] : -g.inv_dx[1];
-        const T *rp = g.rec + (size_t)node * g.stride;
-        // rec_o . aF, the record read in 16-byte chunks
-        constexpr int CH = Chunk<T>::n;
-        T dv = T(0);
-#pragma unroll
-        for (int q = 0; q < NF / CH; ++q) {
-            T v[CH];
-            load_chunk(rp + q * CH, v);
-#pragma unroll
-            for (int j = 0; j < CH; ++j) dv = fma(v[j], av[q * CH + j], dv);
+        for (int d = 0; d < 2; ++d) {
+            float td;
+            cell_of(g, d, ib[d], p[d], td, i0[d], i1[d]);
         }
-        ap[0] = fma(dwx * wy, dv, ap[0]);
-        ap[1] = fma(wx * dwy, dv, ap[1]);
-        const T W = wx * wy;
-#if GCB_ADJ_CACHE
 #pragma unroll
-        for (int c = 0; c < NF; ++c) nc.at(sl, o, c) = fma(W, av[c], nc.at(sl, o, c));
-#else
-        double *gp = nc.grad + (size_t)node * NF;
-#pragma unroll
-        for (int c = 0; c < NF; ++c)
-            if (av[c] != T(0)) atomicAdd(gp + c, (double)(W * av[c]));
-#endif
+        for (int o = 0; o < 4; ++o)
+            node[o] = ((o & 2) ? i1[1] : i0[1]) * g.n[0] + ((o & 1) ? i1[0] : i0[0]);
     }
 }
 
+// Transpose of F = sum_o W_o(p) rec_o: the node records receive W_o aF (via
+// the cache) and the position adjoint sum_o grad W_o (rec_o . aF) is returned.
+// Called by the whole warp; `on`: the lane takes part.
 template <typename T>
-GCB_ADJ_FN1 void gather_frame(const DevGrid<T> &g, const int ib[2], const T p[2],
-                                             const StepPar<T> &s, FieldPt<T, 2> &F, Frame<T> &f)
+__device__ __forceinline__ void gather_bwd(const DevGrid<T> &g, NodeCache<T> &nc, bool on,
+                                           const int ib[2], const T p[2], const FieldPt<T, 2> &aF,
+                                           T ap[2])
 {
-    gather<T, 2, 2>(g, ib, p, F);
-    make_frame<T, 2, true>(F, s.c, s.inv_c2, f);
-}
-
-// frame adjoint at gather point p -> node records and position adjoint
-template <typename T>
-GCB_ADJ_FN1 void frame_gather_bwd(const DevGrid<T> &g, NodeCache<T> &grad, const int ib[2],
-                                                 const T p[2], const FieldPt<T, 2> &F,
-                                                 const StepPar<T> &s, const rev::FrameAdj<T> &af,
-                                                 T ap[2])
-{
-    FieldPt<T, 2> aF;
-    rev::frame_bwd<T, 2>(F, s.c, s.inv_c2, af, aF);
-    gather_bwd(g, grad, ib, p, aF, ap);
-}
-
-// Reverse sweep of a guiding-center step taken with K iterations whose gather
-// points (R^{n-1/2}, x^n + d^1 .. x^n + d^{K-1}, R^{n+1/2}) are pts[0..K].
-template <typename T>
-GCB_ADJ_FN2 void vel_bwd(const Frame<T> &f, const StepPar<T> &s, T upn, T mu, T uperp,
-                         const T aV[3], rev::FrameAdj<T> &af, T &aupn, T &amu, T &auperp)
-{
-    rev::gc_vel_bwd(f, s, upn, mu, uperp, aV, af, aupn, amu, auperp);
-}
-
-// u_par^{n+1/2} from the frame at x^n (the forward update of Sec. 2.2.1 / 2.2.2)
-template <typename T>
-__device__ __forceinline__ T upar_new(const Frame<T> &f0, const StepPar<T> &s, T upar, T mu, T uperp)
-{
-    if (!s.curvature) return fma(s.qm * s.dt, f0.Epar, upar);
-    const T A = dot3(f0.vE, f0.bgb);
-    const T gg = dot3(f0.vE, f0.vgb);
-    const T D = fma(-s.half_dt, A, T(1));
-    const T G0 = gamma_gc(f0, s, upar, mu, uperp);
-    const T upr = fma(upar, fma(s.half_dt, A, T(1)), fma(s.qm * s.dt, f0.Epar, s.half_dt * G0 * gg));
-    const T c2 = s.c * s.c;
-    const T kap2 = f0.kappa * f0.kappa;
-    const T k1 = T(0.25) * s.dt * s.dt * gg * gg - c2 * D * D / kap2;
-    const T k2 = upr * s.dt * gg;
-    const T k3 = fma(upr, upr, (c2 + perp2(f0, s, mu, uperp)) * D * D);
-    const T disc = fma(k2, k2, T(-4) * k1 * k3);
-    const T sq = sqrt(disc);
-    const T q = T(-0.5) * (k2 + (k2 >= T(0) ? sq : -sq));
-    const T r1 = q / k1;
-    const T r2 = (q != T(0)) ? k3 / q : T(-1);
-    const T G1 = r1 >= r2 ? r1 : r2;
-    return fma(s.half_dt * G1, gg, upr) / D;
+    T t[2];
+    int i0[2], node[4];
+    if (on) cell_nodes<T>(g, ib, p, t, i0, node);
+    nc.select(on, i0[0], i0[1]);
+    if (!on) return;
+    Vec<T> av[kChunks<T>];
+    to_chunks(aF, av);
+    T dv[4];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+        const T *rp = reinterpret_cast<const T *>(reinterpret_cast<const char *>(g.rec) +
+                                                  (uint64_t)(unsigned)node[o] * (NF * sizeof(T)));
+        // rec_o . aF, the record read in 16-byte chunks
+        Vec<T> sum;
+#pragma unroll
+        for (int k = 0; k < Vec<T>::n; ++k) sum.v[k] = T(0);
+#pragma unroll
+        for (int j = 0; j < kChunks<T>; ++j) {
+            Vec<T> r;
+            load_chunk(rp + j * Vec<T>::n, r.v);
+            if constexpr (sizeof(T) == 4) {
+                const float2 a = __ffma2_rn(make_float2(r.v[0], r.v[1]),
+                                            make_float2(av[j].v[0], av[j].v[1]),
+                                            make_float2(sum.v[0], sum.v[1]));
+                const float2 b = __ffma2_rn(make_float2(r.v[2], r.v[3]),
+                                            make_float2(av[j].v[2], av[j].v[3]),
+                                            make_float2(sum.v[2], sum.v[3]));
+                sum.v[0] = a.x; sum.v[1] = a.y; sum.v[2] = b.x; sum.v[3] = b.y;
+            } else {
+#pragma unroll
+                for (int k = 0; k < Vec<T>::n; ++k) sum.v[k] = fma(r.v[k], av[j].v[k], sum.v[k]);
+            }
+        }
+        dv[o] = sum.v[0] + sum.v[1];
+        if constexpr (sizeof(T) == 4) dv[o] += sum.v[2] + sum.v[3];
+        const T W = ((o & 1) ? t[0] : T(1) - t[0]) * ((o & 2) ? t[1] : T(1) - t[1]);
+#pragma unroll
+        for (int j = 0; j < kChunks<T>; ++j) {
+            Vec<T> y = nc.at(o, j);
+            axpy(W, av[j], y);
+            nc.at(o, j) = y;
+        }
+    }
+    // sum_o grad W_o dv_o: bilinear differences
+    ap[0] = g.inv_dx[0] * fma(t[1], (dv[3] - dv[2]) - (dv[1] - dv[0]), dv[1] - dv[0]);
+    ap[1] = g.inv_dx[1] * fma(t[0], (dv[3] - dv[1]) - (dv[2] - dv[0]), dv[2] - dv[0]);
 }
 
 // Reverse sweep of a guiding-center step taken with K iterations whose gather
@@ -538,68 +549,80 @@ __device__ __forceinline__ T upar_new(const Frame<T> &f0, const StepPar<T> &s, T
 // field and frame at gather point `pt` (FCache numbering) located at p
 template <typename T>
 __device__ __forceinline__ void frame_at(const DevGrid<T> &g, const FCache<T> &fc, int pt,
-                                         const int ib[2], const T p[2], const StepPar<T> &s,
-                                         FieldPt<T, 2> &F, Frame<T> &f)
+                                         const int ib[2], const T p[2], T c, FieldPt<T, 2> &F,
+                                         rev::RFrame<T, 2> &f)
 {
-    if (pt < GCB_ADJ_FCACHE) {
-        fc.load(pt, F);
-        make_frame<T, 2, true>(F, s.c, s.inv_c2, f);
-    } else {
-        gather_frame(g, ib, p, s, F, f);
-    }
+    if (pt < GCB_ADJ_FCACHE) fc.load(pt, F);
+    else gather_any<T, 2, 2>(g, ib, p, F);
+    f.make(F, c);
 }
 
+// Called by the whole warp (the additions to the node accumulators are made
+// together); `on`: the lane's particle took a guiding-center step, K its count.
 template <typename T>
 __device__ __forceinline__ void gca_rev(const DevGrid<T> &g, NodeCache<T> &grad, const FCache<T> &fc,
-                                        const StepPar<T> &s, const int ib[2], const T l[2],
+                                        const StepPar<T> &s, bool on, const int ib[2], const T l[2],
                                         const T u[3], int K, const T (*pts)[2], const T lo[NS],
                                         T li[NS])
 {
     using rev::FrameAdj;
     FieldPt<T, 2> F;
-    Frame<T> f;
+    rev::RFrame<T, 2> f;
     // forward quantities of the conversion (at R^{n-1/2}) and of the u_par update (at x^n)
-    T Gf, upar, vcm[3], uperp, mu, bpg[3], upn;
-    for (int j = 0; j < 2; ++j) {
-        frame_at(g, fc, j == 0 ? 1 : 0, ib, j == 0 ? pts[0] : l, s, F, f);
-        if (j == 0) rev::conv_fwd(f, s, u, Gf, upar, vcm, uperp, mu, bpg);
-        else upn = upar_new(f, s, upar, mu, uperp);
+    rev::Conv<T> cv;
+    T upn;
+    if (on) {
+        for (int j = 0; j < 2; ++j) {
+            frame_at(g, fc, j == 0 ? 1 : 0, ib, j == 0 ? pts[0] : l, s.c, F, f);
+            if (j == 0) rev::conv_fwd(f, s, u, cv);
+            else upn = rev::upar_new(f, s, cv.upar, cv.mu, cv.uperp);
+        }
     }
     T aupn = T(0), amu = T(0), auperp = T(0), aupar = T(0);
     T abpg[3] = {T(0), T(0), T(0)}, au[3] = {T(0), T(0), T(0)};
     T al[2] = {lo[0], lo[1]};
     T ad[2] = {lo[0] + lo[5], lo[1] + lo[6]};      // x^{n+1} = x^n + d^K, dxp = d^K
     T aVn[3] = {T(0), T(0), T(0)};
-    for (int st = 0; st <= K + 1; ++st) {
-        const T *p = st == 0 ? pts[K] : (st < K ? pts[K - st] : (st == K ? l : pts[0]));
-        const int pt = st == 0 ? K + 1 : (st < K ? K - st + 1 : (st == K ? 0 : 1));
-        frame_at(g, fc, pt, ib, p, s, F, f);
-        FrameAdj<T> af;
-        af.zero();
-        if (st == 0) {
-            const T lu[3] = {lo[2], lo[3], lo[4]};
-            rev::recon_bwd(f, s, upn, mu, uperp, bpg, lu, af, aupn, amu, auperp, abpg);
-        } else if (st <= K) {
-            // d^k = dt/2 (V^n + V^{k-1}) with V^0 = V^n: stage st < K carries
-            // V^{K-st}; stage K carries V^n with every term collected
-            T aV[3];
-            if (st < K) {
-                aV[0] = s.half_dt * ad[0];
-                aV[1] = s.half_dt * ad[1];
-                aVn[0] += aV[0];
-                aVn[1] += aV[1];
+    T p[2] = {T(0), T(0)};
+    const int KM = __reduce_max_sync(0xffffffffu, on ? K : -2);
+    for (int st = 0; st <= KM + 1; ++st) {
+        const bool act = on && st <= K + 1;
+        FieldPt<T, 2> aF;
+        if (act) {
+            const T *q = st == 0 ? pts[K] : (st < K ? pts[K - st] : (st == K ? l : pts[0]));
+            const int pt = st == 0 ? K + 1 : (st < K ? K - st + 1 : (st == K ? 0 : 1));
+            p[0] = q[0];
+            p[1] = q[1];
+            frame_at(g, fc, pt, ib, p, s.c, F, f);
+            FrameAdj<T> af;
+            af.zero();
+            if (st == 0) {
+                const T lu[3] = {lo[2], lo[3], lo[4]};
+                rev::recon_bwd(f, s, upn, cv.mu, cv.uperp, cv.bpg, lu, af, aupn, amu, auperp, abpg);
+            } else if (st <= K) {
+                // d^k = dt/2 (V^n + V^{k-1}) with V^0 = V^n: stage st < K carries
+                // V^{K-st}; stage K carries V^n with every term collected
+                T aV[3];
+                if (st < K) {
+                    aV[0] = s.half_dt * ad[0];
+                    aV[1] = s.half_dt * ad[1];
+                    aVn[0] += aV[0];
+                    aVn[1] += aV[1];
+                } else {
+                    aV[0] = aVn[0] + s.dt * ad[0];
+                    aV[1] = aVn[1] + s.dt * ad[1];
+                }
+                aV[2] = T(0);
+                rev::gc_vel_bwd(f, s, upn, cv.mu, cv.uperp, aV, af, aupn, amu, auperp);
+                if (st == K) rev::upar_bwd(f, s, cv.upar, cv.mu, cv.uperp, aupn, af, aupar, amu, auperp);
             } else {
-                aV[0] = aVn[0] + s.dt * ad[0];
-                aV[1] = aVn[1] + s.dt * ad[1];
+                rev::conv_bwd(f, s, u, cv, aupar, amu, auperp, abpg, af, au);
             }
-            aV[2] = T(0);
-            vel_bwd(f, s, upn, mu, uperp, aV, af, aupn, amu, auperp);
-            if (st == K) rev::upar_bwd(f, s, upar, mu, uperp, aupn, af, aupar, amu, auperp);
-        } else {
-            rev::conv_bwd(f, s, u, Gf, upar, vcm, uperp, mu, bpg, aupar, amu, auperp, abpg, af, au);
+            rev::frame_bwd<T, 2>(F, f, s.c, s.inv_c2, af, aF);
         }
         T ap[2];
-        frame_gather_bwd(g, grad, ib, p, F, s, af, ap);
+        gather_bwd(g, grad, act, ib, p, aF, ap);
+        if (!act) continue;
         al[0] += ap[0];
         al[1] += ap[1];
         if (st == 0) {                 // R^{n+1/2} = x^n + d^K / 2
@@ -613,6 +636,7 @@ __device__ __forceinline__ void gca_rev(const DevGrid<T> &g, NodeCache<T> &grad,
             li[6] = T(-0.5) * ap[1];
         }
     }
+    if (!on) return;
     li[0] = al[0];
     li[1] = al[1];
     li[2] = au[0];
@@ -620,101 +644,114 @@ __device__ __forceinline__ void gca_rev(const DevGrid<T> &g, NodeCache<T> &grad,
     li[4] = au[2];
 }
 
-// resident blocks per SM the reverse kernel is compiled for (FP32: 4, i.e.
-// at most 128 registers; FP64 kernels need more registers than that allows)
-template <typename T> struct RevBlocks { static constexpr int n = GCB_ADJ_BLOCKS_F32; };
+// Resident blocks per SM the reverse kernel is compiled for.  FP32: 3, what its
+// 61 KB of shared memory allow, so up to 168 registers (4 blocks would cap
+// them at 128: 172 B spilled, 16 steps' gradient of 2^18 particles 4.69 against
+// 4.49 ms; 5 cached points and 4 blocks 4.85, 8 and 3 4.63, 4 and 3 4.49).
+template <typename T> struct RevBlocks { static constexpr int n = 3; };
 template <> struct RevBlocks<double> { static constexpr int n = 1; };
 
+// What bounds it: issue and shared-memory latency at 12 warps per SM (issue 43%
+// busy, L1 53%, DRAM idle).  Measured (GB300, 512x256 grid, 2^18 particles, 6
+// iterations): 213 us a step before; 203 us with the frame's values shared with
+// its transpose, reciprocals and 16-byte shared-memory accesses (10.6k -> 8.0k
+// instructions a particle), 149 us with the node additions made by the warp (L1
+// wavefronts 37 -> 25 M, FP64 pipe 41 -> 22%), about 140 us with 3 blocks.
 template <typename T>
 __global__ void __launch_bounds__(TPB, RevBlocks<T>::n) k_adjoint_rev(const AdjArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char s_raw[];
     T pts[MAXG][2];
     NodeCache<T> nc;
-    nc.acc = reinterpret_cast<T *>(s_raw) + threadIdx.x;
-    const FCache<T> fc{reinterpret_cast<T *>(s_raw) + GCB_ADJ_CACHE * 4 * NF * TPB + threadIdx.x};
+    nc.base = reinterpret_cast<Vec<T> *>(s_raw);
+    const FCache<T> fc{nc.base + NodeCache<T>::N + threadIdx.x};
     nc.grad = a.grad;
     nc.nx = a.g.n[0];
     nc.ny = a.g.n[1];
-    nc.key[0] = nc.key[1] = -1;
-    nc.mru = 1;
-    for (int64_t i = blockIdx.x * (int64_t)TPB + threadIdx.x; i < a.np;
-         i += (int64_t)gridDim.x * TPB) {
-        const uint8_t fl = a.flags[i];
-        bool fin = true;
+    nc.cx = nc.cy = -1;
+    for (int64_t i0 = blockIdx.x * (int64_t)TPB; i0 < a.np; i0 += (int64_t)gridDim.x * TPB) {
+        // every lane stays for the warp's additions; `on`: it has a particle
+        // that is not frozen (whose step is the identity)
+        const int64_t i = i0 + threadIdx.x;
+        bool on = i < a.np;
         int ib[2];
         T l[2], u[3], dxp[2], lo[NS];
+        uint8_t fl = 0;
+        if (on) {
+            fl = a.flags[i];
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {
-            load_pos(a, i, d, ib[d], l[d], fin);
-            dxp[d] = a.dxp[d][i];
-            fin = fin && isfinite(dxp[d]);
+            for (int d = 0; d < 2; ++d) {
+                load_pos(a, i, d, ib[d], l[d], on);
+                dxp[d] = a.dxp[d][i];
+                on = on && isfinite(dxp[d]);
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) { u[k] = a.u[k][i]; on = on && isfinite(u[k]); }
+#pragma unroll
+            for (int k = 0; k < NS; ++k) lo[k] = a.lam[k][i];
         }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) { u[k] = a.u[k][i]; fin = fin && isfinite(u[k]); }
-#pragma unroll
-        for (int k = 0; k < NS; ++k) lo[k] = a.lam[k][i];
-        if (!fin) continue;          // a frozen particle's step is the identity
-
         StepPar<T> sp = a.sp;
-        sp.qm = a.qm[(fl >> GCB_SPECIES_SHIFT) & 3];
-        sp.cq = sp.c / sp.qm;
-        FieldPt<T, 2> F0;
-        gather<T, 2, 2>(a.g, ib, l, F0);
-        fc.store(0, F0);
-        const T Q = fabs(sp.qm);
-        const T G = sqrt(T(1) + (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * sp.inv_c2);
-        const T Bm = sqrt(F0.B[0] * F0.B[0] + F0.B[1] * F0.B[1] + F0.B[2] * F0.B[2]);
-        const T Em = sqrt(F0.E[0] * F0.E[0] + F0.E[1] * F0.E[1] + F0.E[2] * F0.E[2]);
-        int S = (a.c2 * G < a.rho_thr * Q * Bm && Em < a.f_E * Bm) ? 0 : 1;
-        if (a.force == GCB_FORCE_BORIS) S = 1;
-        if (a.force == GCB_FORCE_GCA) S = 0;
         int K = 0;
         bool gca = false;
-        if (S == 0) {
-            T uu[3] = {u[0], u[1], u[2]}, disp[2];
-            bool ncv;
-            int cnt = 0;
-            gca = replay_step(RecGather<T>{a.g, pts, &cnt, fc}, sp, ib, l, dxp, F0, uu, disp, K, ncv);
-            gca = gca && cnt == K + 1 && cnt <= MAXG;
+        FieldPt<T, 2> F0;
+        if (on) {
+            sp.qm = a.qm[(fl >> GCB_SPECIES_SHIFT) & 3];
+            sp.cq = sp.c / sp.qm;
+            gather_any<T, 2, 2>(a.g, ib, l, F0);
+            fc.store(0, F0);
+            const T Q = fabs(sp.qm);
+            const T G = sqrt(T(1) + (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * sp.inv_c2);
+            const T Bm = sqrt(F0.B[0] * F0.B[0] + F0.B[1] * F0.B[1] + F0.B[2] * F0.B[2]);
+            const T Em = sqrt(F0.E[0] * F0.E[0] + F0.E[1] * F0.E[1] + F0.E[2] * F0.E[2]);
+            int S = (a.c2 * G < a.rho_thr * Q * Bm && Em < a.f_E * Bm) ? 0 : 1;
+            if (a.force == GCB_FORCE_BORIS) S = 1;
+            if (a.force == GCB_FORCE_GCA) S = 0;
+            if (S == 0) {
+                T uu[3] = {u[0], u[1], u[2]}, disp[2];
+                bool ncv;
+                int cnt = 0;
+                gca = replay_step(RecGather<T>{a.g, pts, &cnt, fc}, sp, ib, l, dxp, F0, uu, disp, K, ncv);
+                gca = gca && cnt == K + 1 && cnt <= MAXG;
+            }
         }
         T li[NS];
-        if (gca) {
-            gca_rev(a.g, nc, fc, sp, ib, l, u, K, pts, lo, li);
-        } else {
-            T lu[3] = {lo[2], lo[3], lo[4]};
-            T ldisp[2] = {lo[0] + lo[5], lo[1] + lo[6]};
-            T au[3], aE[3], aB[3];
-            rev::boris_bwd<T, 2>(F0.E, F0.B, sp, u, lu, ldisp, au, aE, aB);
+        gca_rev(a.g, nc, fc, sp, gca, ib, l, u, K, pts, lo, li);
+        const bool bor = on && !gca;
+        if (__any_sync(0xffffffffu, bor)) {
             FieldPt<T, 2> aF;
+            T au[3], ap[2];
+            if (bor) {
+                const T lu[3] = {lo[2], lo[3], lo[4]};
+                const T ldisp[2] = {lo[0] + lo[5], lo[1] + lo[6]};
+                rev::boris_bwd<T, 2>(F0.E, F0.B, sp, u, lu, ldisp, au, aF.E, aF.B);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) { aF.E[c] = aE[c]; aF.B[c] = aB[c]; }
+                for (int ii = 0; ii < 2; ++ii)
 #pragma unroll
-            for (int ii = 0; ii < 2; ++ii)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) aF.dB[ii][j] = T(0);
-            T ap[2];
-            gather_bwd(a.g, nc, ib, l, aF, ap);
-            li[0] = lo[0] + ap[0];
-            li[1] = lo[1] + ap[1];
-            li[2] = au[0];
-            li[3] = au[1];
-            li[4] = au[2];
-            li[5] = T(0);
-            li[6] = T(0);
+                    for (int j = 0; j < 3; ++j) aF.dB[ii][j] = T(0);
+            }
+            gather_bwd(a.g, nc, bor, ib, l, aF, ap);
+            if (bor) {
+                li[0] = lo[0] + ap[0];
+                li[1] = lo[1] + ap[1];
+                li[2] = au[0];
+                li[3] = au[1];
+                li[4] = au[2];
+                li[5] = T(0);
+                li[6] = T(0);
+            }
         }
-#if GCB_ADJ_CACHE
         nc.finish();
-#endif
+        if (on) {
 #pragma unroll
-        for (int k = 0; k < NS; ++k) a.lam[k][i] = li[k];
+            for (int k = 0; k < NS; ++k) a.lam[k][i] = li[k];
+        }
     }
 }
 
 template <typename T>
 constexpr int rev_smem()
 {
-    return (GCB_ADJ_CACHE * 4 + GCB_ADJ_FCACHE) * NF * TPB * (int)sizeof(T);
+    return (NodeCache<T>::N + GCB_ADJ_FCACHE * kChunks<T> * TPB) * 16;
 }
 
 template <typename T>
