@@ -843,38 +843,129 @@ gcb_status adjoint_step(const gcb_particles *s, const gcb_grid *g, const gcb_par
 namespace gcb {
 namespace adj {
 
-// dL/da_m = sum_e grad[e] pat_m[e]; grid row m = blockIdx.y.
-template <typename PT>
-__global__ void __launch_bounds__(256) k_project(const double *grad, const PT *pat, int64_t nelem,
-                                                 double *out)
+// Both kernels take one FP64 multiply-add per pattern value, which the FP64 pipe
+// bounds (2^17 nodes, 64 modes: 100.7 M, 160 us; the patterns' 403 MB take 60
+// us).  Values are read V at a time (16 bytes; V = 1 where a pointer is not
+// 16-byte aligned) and widened by their bits, which keeps the conversions off
+// that pipe.  Measured (GB300, FP32 patterns): combination 382 -> 190 us,
+// projection 481 -> 195 us (FP64 patterns 194 -> 178 and 288 -> 268 us).
+template <typename PT, int V>
+struct Pack { PT v[V]; };
+template <typename PT, int V>
+__device__ __forceinline__ Pack<PT, V> load_pack(const PT *p)
 {
-    __shared__ double s_w[8];
-    const int m = blockIdx.y;
-    const PT *pm = pat + (size_t)m * nelem;
-    double acc = 0.0;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nelem;
-         e += (int64_t)gridDim.x * blockDim.x)
-        acc = fma(grad[e], (double)pm[e], acc);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = acc;
+    Pack<PT, V> r;
+    if constexpr (V == 1) r.v[0] = __ldg(p);
+    else load_chunk(p, r.v);
+    return r;
+}
+
+// dL/da_m = sum_e grad[e] pat_m[e]: a thread takes MB modes (grid row: modes
+// MB blockIdx.y ...), so that grad is read once and the block's sums are
+// reduced once for MB of them.
+constexpr int MB = 8;
+template <typename PT, int V>
+__global__ void __launch_bounds__(256) k_project(const double *grad, const PT *pat, int64_t nelem,
+                                                 int nmodes, double *out)
+{
+    __shared__ double s_w[8][MB];
+    const int m0 = blockIdx.y * MB;
+    double acc[MB];
+#pragma unroll
+    for (int j = 0; j < MB; ++j) acc[j] = 0.0;
+    for (int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * V; e < nelem;
+         e += (int64_t)gridDim.x * blockDim.x * V) {
+        double g[V];
+        if constexpr (V == 1) {
+            g[0] = grad[e];
+        } else {
+#pragma unroll
+            for (int k = 0; k < V; k += 2) load_chunk(grad + e + k, g + k);
+        }
+        Pack<PT, V> r[MB];
+#pragma unroll
+        for (int j = 0; j < MB; ++j)   // past the last mode: mode m0 again, not added
+            r[j] = load_pack<PT, V>(pat + (size_t)(m0 + j < nmodes ? m0 + j : m0) * nelem + e);
+#pragma unroll
+        for (int j = 0; j < MB; ++j)
+            if (m0 + j < nmodes)
+#pragma unroll
+                for (int k = 0; k < V; ++k) acc[j] = fma(g[k], widen<true>(r[j].v[k]), acc[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < MB; ++j) {
+        for (int o = 16; o > 0; o >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
+        if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5][j] = acc[j];
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < MB && m0 + (int)threadIdx.x < nmodes) {
         double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_w[w];
-        atomicAdd(&out[m], t);
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_w[w][threadIdx.x];
+        atomicAdd(&out[m0 + threadIdx.x], t);
     }
 }
 
-template <typename PT>
-__global__ void k_combine(PT *rec, const PT *base, const PT *pat, const double *amps, int64_t nelem,
-                          int nmodes)
+// rec = base + sum_m amps[m] pat_m
+template <typename PT, int V>
+__global__ void __launch_bounds__(256) k_combine(PT *rec, const PT *base, const PT *pat,
+                                                 const double *amps, int64_t nelem, int nmodes)
 {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nelem;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        double v = (double)base[e];
-        for (int m = 0; m < nmodes; ++m) v = fma(amps[m], (double)pat[(size_t)m * nelem + e], v);
-        rec[e] = (PT)v;
+    for (int64_t e = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * V; e < nelem;
+         e += (int64_t)gridDim.x * blockDim.x * V) {
+        double v[V];
+        const Pack<PT, V> b = load_pack<PT, V>(base + e);
+#pragma unroll
+        for (int k = 0; k < V; ++k) v[k] = widen<true>(b.v[k]);
+#pragma unroll 8
+        for (int m = 0; m < nmodes; ++m) {
+            const Pack<PT, V> r = load_pack<PT, V>(pat + (size_t)m * nelem + e);
+            const double w = __ldg(amps + m);
+#pragma unroll
+            for (int k = 0; k < V; ++k) v[k] = fma(w, widen<true>(r.v[k]), v[k]);
+        }
+        if constexpr (V == 1) {
+            rec[e] = (PT)v[0];
+        } else {
+            Vec<PT> w;             // the records are 16-byte aligned
+#pragma unroll
+            for (int k = 0; k < V; ++k) w.v[k] = (PT)v[k];
+            *reinterpret_cast<Vec<PT> *>(rec + e) = w;
+        }
     }
+}
+
+static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
+// (nelem is a multiple of a record's 16-byte chunks, so every mode's values
+// are aligned as the first one's)
+template <typename PT>
+static void launch_project(const double *grad, const PT *pat, int64_t nelem, int nmodes, double *out,
+                           cudaStream_t st)
+{
+    const int groups = (nmodes + MB - 1) / MB;
+    auto blocks = [&](int v) {
+        int64_t n = (nelem / v + 255) / 256, cap = 152 * 6 / groups;
+        return (unsigned)(n < cap ? n : cap);
+    };
+    constexpr int V = Chunk<PT>::n;
+    if (aligned16(grad) && aligned16(pat))
+        k_project<PT, V><<<dim3(blocks(V), groups), 256, 0, st>>>(grad, pat, nelem, nmodes, out);
+    else
+        k_project<PT, 1><<<dim3(blocks(1), groups), 256, 0, st>>>(grad, pat, nelem, nmodes, out);
+}
+template <typename PT>
+static void launch_combine(PT *rec, const PT *base, const PT *pat, const double *amps, int64_t nelem,
+                           int nmodes, cudaStream_t st)
+{
+    auto blocks = [&](int v) {
+        const int64_t n = (nelem / v + 255) / 256;
+        return (unsigned)(n < 152 * 32 ? n : 152 * 32);
+    };
+    constexpr int V = Chunk<PT>::n;
+    if (aligned16(base) && aligned16(pat))
+        k_combine<PT, V><<<blocks(V), 256, 0, st>>>(rec, base, pat, amps, nelem, nmodes);
+    else
+        k_combine<PT, 1><<<blocks(1), 256, 0, st>>>(rec, base, pat, amps, nelem, nmodes);
 }
 
 }  // namespace adj
@@ -887,13 +978,10 @@ gcb_status grad_project(const gcb_grid *g, const double *grad, const void *pat, 
         set_error("cudaMemsetAsync: %s", cudaGetErrorString(cudaGetLastError()));
         return GCB_ECUDA;
     }
-    int64_t nb = (nelem + 255) / 256;
-    if (nb > 152 * 4) nb = 152 * 4;
-    const dim3 grid((unsigned)nb, (unsigned)nmodes);
     if (g->dtype == GCB_F32)
-        adj::k_project<float><<<grid, 256, 0, st>>>(grad, (const float *)pat, nelem, out);
+        adj::launch_project<float>(grad, (const float *)pat, nelem, nmodes, out, st);
     else
-        adj::k_project<double><<<grid, 256, 0, st>>>(grad, (const double *)pat, nelem, out);
+        adj::launch_project<double>(grad, (const double *)pat, nelem, nmodes, out, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { set_error("k_project: %s", cudaGetErrorString(e)); return GCB_ECUDA; }
     return GCB_OK;
@@ -903,14 +991,12 @@ gcb_status grid_combine(const gcb_grid *g, const void *base, const void *pat, co
                         int nmodes, cudaStream_t st)
 {
     const int64_t nelem = g->n[0] * g->n[1] * g->n[2] * (int64_t)g->stride;
-    int64_t nb = (nelem + 255) / 256;
-    if (nb > 152 * 32) nb = 152 * 32;
     if (g->dtype == GCB_F32)
-        adj::k_combine<float><<<(int)nb, 256, 0, st>>>((float *)g->rec, (const float *)base,
-                                                       (const float *)pat, amps, nelem, nmodes);
+        adj::launch_combine<float>((float *)g->rec, (const float *)base, (const float *)pat, amps,
+                                   nelem, nmodes, st);
     else
-        adj::k_combine<double><<<(int)nb, 256, 0, st>>>((double *)g->rec, (const double *)base,
-                                                        (const double *)pat, amps, nelem, nmodes);
+        adj::launch_combine<double>((double *)g->rec, (const double *)base, (const double *)pat, amps,
+                                    nelem, nmodes, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { set_error("k_combine: %s", cudaGetErrorString(e)); return GCB_ECUDA; }
     return GCB_OK;

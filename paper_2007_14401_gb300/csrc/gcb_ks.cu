@@ -199,17 +199,6 @@ __device__ __forceinline__ void ks_cell(const KsGrid<FT> &g, double lr, double t
     ks_axis(th * g.inv_dth, g.nth - 1, j, tt);
 }
 
-// A float as a double, by its bits: the conversion instruction would take an
-// FP64 pipe slot (zeros, denormals, infinities and NaN go through it).
-__device__ __forceinline__ double widen(float f)
-{
-    const unsigned b = __float_as_uint(f), e = (b >> 23) & 0xffu;
-    if (e - 1u >= 0xfeu) return (double)f;
-    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)),
-                            (int)(b << 29));
-}
-__device__ __forceinline__ double widen(double f) { return f; }
-
 // linear-shape-function gather of D^i, B^i (Sec. 4 intro) in the record type
 // (lr: log r)
 template <typename FT>
@@ -230,7 +219,7 @@ __device__ __forceinline__ void ks_gather(const KsGrid<FT> &g, double lr, double
         for (int k = 0; k < 6; ++k) acc[k] = fma(__ldg(rp + k), W, acc[k]);
     }
 #pragma unroll
-    for (int k = 0; k < 3; ++k) { D[k] = widen(acc[k]); B[k] = widen(acc[3 + k]); }
+    for (int k = 0; k < 3; ++k) { D[k] = widen<false>(acc[k]); B[k] = widen<false>(acc[3 + k]); }
 }
 
 __device__ __forceinline__ void cross(const double a[3], const double b[3], double x[3])

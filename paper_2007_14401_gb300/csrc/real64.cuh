@@ -61,6 +61,25 @@ __device__ __forceinline__ double sqrt64(double x)
     return not_pos_normal(x) && __double2hiint(x) >= 0 ? x : r;
 }
 
+// A float as a double, by its bits: the conversion instruction takes an FP64
+// pipe slot.  Denormals: flushed to zero (FTZ, as the conversion does in the
+// units compiled with that flag), else converted by the instruction (the asm is
+// volatile, so that it is not issued for every value and then selected).
+template <bool FTZ>
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned b = __float_as_uint(f), a = b & 0x7fffffffu;
+    const bool norm = a >= 0x00800000u;
+    // exponent bias 1023 - 127; infinities and NaN to the top exponent
+    const unsigned h = (a >> 3) + (a >= 0x7f800000u ? 0x70000000u : 0x38000000u);
+    double r = __hiloint2double((int)((b & 0x80000000u) | (norm ? h : 0u)),
+                                (int)(norm ? b << 29 : 0u));
+    if (!FTZ && a - 1u < 0x007fffffu) asm volatile("cvt.f64.f32 %0, %1;" : "=d"(r) : "f"(f));
+    return r;
+}
+template <bool FTZ>
+__device__ __forceinline__ double widen(double f) { return f; }
+
 // floor(s): its value, and as an integer clamped to [-n, n].  Adding 1.5 2^52
 // rounded down leaves the floor in the low bits of the sum (exact for
 // |s| < 2^51; beyond, and for NaN, the integer clamps).  2 FP64 additions in
