@@ -314,7 +314,7 @@ __device__ __forceinline__ void interp_cell(const DevGrid<float> &g, const CellR
     float2 acc[NP];
 #pragma unroll
     for (int k = 0; k < NP; ++k) acc[k] = make_float2(0.f, 0.f);
-    float2 dacc[ND][2];                          // grad-W mode: d_i (B0,B1), d_i (B2,-)
+    float2 dacc[ND][2];                          // grad-W mode: d_i (-,B0), d_i (B1,B2), as loaded
     if (GM == 1) {
 #pragma unroll
         for (int i = 0; i < ND; ++i) dacc[i][0] = dacc[i][1] = make_float2(0.f, 0.f);
@@ -331,9 +331,6 @@ __device__ __forceinline__ void interp_cell(const DevGrid<float> &g, const CellR
 #pragma unroll
         for (int k = 0; k < NP; ++k) acc[k] = __ffma2_rn(cr.pr[o][k], W2, acc[k]);
         if (GM == 1) {
-            // pairs 1 and 2 hold (E2, B0) and (B1, B2)
-            const float2 b01 = make_float2(cr.pr[o][1].y, cr.pr[o][2].x);
-            const float2 b2 = make_float2(cr.pr[o][2].y, 0.f);
 #pragma unroll
             for (int i = 0; i < ND; ++i) {
                 float gw = ((o >> i) & 1) ? g.inv_dx[i] : -g.inv_dx[i];
@@ -341,8 +338,8 @@ __device__ __forceinline__ void interp_cell(const DevGrid<float> &g, const CellR
                 for (int e = 0; e < ND; ++e)
                     if (e != i) gw *= w[e];
                 const float2 G2 = make_float2(gw, gw);
-                dacc[i][0] = __ffma2_rn(b01, G2, dacc[i][0]);
-                dacc[i][1] = __ffma2_rn(b2, G2, dacc[i][1]);
+                dacc[i][0] = __ffma2_rn(cr.pr[o][1], G2, dacc[i][0]);
+                dacc[i][1] = __ffma2_rn(cr.pr[o][2], G2, dacc[i][1]);
             }
         }
     }
@@ -359,9 +356,9 @@ __device__ __forceinline__ void interp_cell(const DevGrid<float> &g, const CellR
     } else if (GM == 1) {
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
-            F.dB[i][0] = dacc[i][0].x;
-            F.dB[i][1] = dacc[i][0].y;
-            F.dB[i][2] = dacc[i][1].x;
+            F.dB[i][0] = dacc[i][0].y;
+            F.dB[i][1] = dacc[i][1].x;
+            F.dB[i][2] = dacc[i][1].y;
         }
     }
 }
