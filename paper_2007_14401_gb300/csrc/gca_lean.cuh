@@ -103,13 +103,31 @@ __device__ __forceinline__ void lean_drift(const FieldPt<R, ND> &F, const LeanFr
     }
 }
 
+// sin and cos of the gyro-phase -num/den, taken in FP64 (the angle reaches
+// Omega_C dt ~ 1e5 rad in strongly magnetized runs): the angle in half turns,
+// wrapped into [-1, 1] (exact for the multiples of 2 removed), then sin and cos
+// of pi times it.  Out of line: an option's code.
+__device__ __forceinline__ double half_turns(double num, double den)
+{
+    const double t = -num / den * 0.31830988618379067;   // 1/pi
+    return fma(-2.0, rint(0.5 * t), t);
+}
+static __device__ __noinline__ void gyro_sincos(double num, double den, float &sn, float &cs)
+{
+    sincospif((float)half_turns(num, den), &sn, &cs);
+}
+static __device__ __noinline__ void gyro_sincos(double num, double den, double &sn, double &cs)
+{
+    sincospi(half_turns(num, den), &sn, &cs);
+}
+
 // The step: arguments and result as gca_step_c.
 template <typename R, int ND, int GM, typename Gth, bool MIR = false>
 __device__ __forceinline__ bool gca_step_lean(const Gth &gth, const StepPar<R> &s, const int ib[ND],
                                               const R ln[ND], const R dxp[ND],
                                               const FieldPt<R, ND> &F0, R u[3], R disp[ND],
                                               int &iters, bool &nonconv,
-                                              const FieldPt<R, ND> *Fh = nullptr, R *vz = nullptr)
+                                              R *vz = nullptr)
 {
     constexpr bool RAW = RawGrad<R, GM>::value;
     R gs[ND];
@@ -124,8 +142,7 @@ __device__ __forceinline__ bool gca_step_lean(const Gth &gth, const StepPar<R> &
     R pt[ND];
 #pragma unroll
     for (int d = 0; d < ND; ++d) pt[d] = fma(R(-0.5), dxp[d], ln[d]);
-    if (Fh) F = *Fh;
-    else gth(ib, pt, F);
+    gth(ib, pt, F);
     lean_frame<R, ND>(F, s.c, f);
     if (!(f0.ok && f.ok)) return false;
     R v[3], ig;
@@ -285,17 +302,10 @@ __device__ __forceinline__ bool gca_step_lean(const Gth &gth, const StepPar<R> &
     if (s.phase) {
         // evolved gyration phase: u_g turns about b by the step's gyro-phase
         // phi = -(q/m) B dt/(c kappa Gamma) (the lab-time rate of the gyration
-        // in the frame drifting with v_E), taken in FP64 (the angle reaches
-        // Omega_C dt ~ 1e5 rad in strongly magnetized runs)
-        const double phi = -(double)s.qm * (double)(f.B2 * f.ib) * (double)s.dt /
-                           ((double)s.c * (double)f.kap * (double)Gp);
-        // the angle in half turns, wrapped into [-1, 1] (exact for the
-        // multiples of 2 removed), then sin and cos of pi times it
-        const double t = phi * 0.31830988618379067;   // 1/pi
-        const double r = fma(-2.0, rint(0.5 * t), t);
+        // in the frame drifting with v_E)
         R sn, cs;
-        if constexpr (sizeof(R) == 4) sincospif((float)r, &sn, &cs);
-        else sincospi(r, &sn, &cs);
+        gyro_sincos((double)s.qm * (double)(f.B2 * f.ib) * (double)s.dt,
+                    (double)s.c * (double)f.kap * (double)Gp, sn, cs);
         R bxd[3];
         cross3(F.B, ug, bxd);
 #pragma unroll

@@ -41,11 +41,14 @@ struct Tile {
 #define GCB_UNIFORM_TILES 1
 #endif
 // minimum resident threads per SM requested from the register allocator:
-// FP32 2D 512 (at most 128 registers a thread); FP32 3D 384 (at most 170
-// registers: 184 unconstrained leaves 256 threads, which measured 16% slower,
-// and 512 spills)
+// FP32 2D 576 (at most 112 registers a thread; 8 steps of 2^24 particles and
+// their sort 8.32 ms at 512, 7.62 at 576, 7.60 at 640, 7.76 at 704, 8.25 at 768;
+// 2^22 with deposition 2.82, 2.68, 2.71, 2.81, 2.96 ms), and 512 in the exact
+// frame, whose longer frame spills 240 B at 112; FP32 3D 384 (at most
+// 170 registers: 184 unconstrained leaves 256 threads, which measured 16%
+// slower, and 512 spills)
 #ifndef GCB_MIN_THREADS_F32_2D
-#define GCB_MIN_THREADS_F32_2D 512
+#define GCB_MIN_THREADS_F32_2D 576
 #endif
 #ifndef GCB_MIN_THREADS_F32_3D
 #define GCB_MIN_THREADS_F32_3D 384
@@ -56,23 +59,18 @@ struct Tile {
 #ifndef GCB_REG2D
 #define GCB_REG2D 1
 #endif
-// 1: phase 1 gathers at R^{n-1/2} = x^n - dxp/2 together with x^n (2D), so
-// that the two gathers' loads are in flight at once
-#ifndef GCB_HOIST_HALF
-#define GCB_HOIST_HALF 1
-#endif
 // FP32 3D with current deposition and gradient records: 256 (the 3D walk
 // spills 684 B at 384); with gradients from W, 384 as without deposition
 // (measured 14% faster than 256 on the 3D sheet)
 #ifndef GCB_MIN_THREADS_F32_3D_DEP_GRID
 #define GCB_MIN_THREADS_F32_3D_DEP_GRID 256
 #endif
-template <typename R, int ND, int GM = 1, bool DEP = false>
+template <typename R, int ND, int GM = 1, bool DEP = false, bool BT = false>
 struct MinBlocks {
     static constexpr int n = sizeof(R) == 8
         ? 1
         : (ND == 3 ? ((DEP && GM == 2) ? GCB_MIN_THREADS_F32_3D_DEP_GRID : GCB_MIN_THREADS_F32_3D)
-                   : GCB_MIN_THREADS_F32_2D) / Tile<R, ND>::n;
+                   : (BT ? 512 : GCB_MIN_THREADS_F32_2D)) / Tile<R, ND>::n;
 };
 
 template <typename R>
@@ -384,7 +382,7 @@ __device__ __forceinline__ bool deposit_path(const PushArgs<R> &a, const int ib[
 // GEN: gca_step_c where gca_lean.cuh would be used (the adjoint's forward run).
 template <typename R, int ND, int PM, int GM, bool FUSE, bool BT = false, bool DEP = false,
           bool MIR = false, bool GEN = false>
-__global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) k_push_sr(const PushArgs<R> a)
+__global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP, BT>::n) k_push_sr(const PushArgs<R> a)
 {
     static_assert(!(DEP && FUSE), "deposition runs in unfused launches");
     constexpr int TPB = Tile<R, ND>::n;
@@ -426,8 +424,6 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
         float xl[ND];
         R l[ND], uu[3], dd[ND];
         FieldPt<R, ND> F;
-        constexpr bool HOIST = GCB_HOIST_HALF && ND == 2;
-        FieldPt<R, ND> Fh;          // fields at R^{n-1/2} (HOIST)
         int ib[ND];
         // the step's arrangement: gca_lean.cuh for the simplified frame in FP64
         // and in FP32 2D, gca_step_c otherwise
@@ -468,12 +464,6 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
                 }
                 if constexpr (GCB_SEED_CACHE && Gth::kCellCache) gather_cached<ND, GM>(a.g, ib, l, F, cr);
                 else Gth{a.g}(ib, l, F);
-                if constexpr (HOIST) {
-                    R ph[ND];
-#pragma unroll
-                    for (int d = 0; d < ND; ++d) ph[d] = fma(R(-0.5), dd[d], l[d]);
-                    Gth{a.g}(ib, ph, Fh);
-                }
                 // switch S (Sec. 3, Sec. 4.1) in division-free form:
                 // S = 0 iff c^2 Gamma < f_rho dl |q/m| B and |E| < f_E B.
                 int S;
@@ -641,12 +631,11 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP>::n) 
             if (isg) {
                 if constexpr (LEAN)
                     done = gca_step_lean<R, ND, GM, Gth, MIR>(Gth{a.g}, sp, ib, l, ds, F, us, disp,
-                                                              it, ncv, (HOIST && uni) ? &Fh : nullptr,
+                                                              it, ncv,
                                                               (DEP && ND == 2) ? &vzg : nullptr);
                 else
                     done = gca_step_c<R, ND, GM, Gth, BT, MIR>(Gth{a.g}, sp, ib, l, ds, F, us, disp, it,
-                                                          ncv, cr, (HOIST && uni) ? &Fh : nullptr,
-                                                          (DEP && ND == 2) ? &vzg : nullptr);
+                                                          ncv, cr, (DEP && ND == 2) ? &vzg : nullptr);
                 if (!done) {
                     fail = true;
                     it = 0;
