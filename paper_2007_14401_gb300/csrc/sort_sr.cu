@@ -1,11 +1,11 @@
 // sort_sr.cu -- counting sort of the particle arrays by tile of cells.
 //
-// keys    : tile index of every particle (row-major over tiles, non-finite
-//           particles in an extra last bucket); the rank inside the bucket
-//           comes from one atomicAdd per group of equal keys in a warp
-//           (__match_any_sync), so runs of already-sorted particles cost one
-//           atomic per warp.
-// scan    : exclusive prefix sum of the bucket counts (multi-block).
+// keys    : tile index of every particle (row-major over tiles, particles with a
+//           non-finite position in an extra last bucket); the rank inside the
+//           bucket comes from one atomicAdd per run of equal keys in a warp,
+//           so runs of already-sorted particles cost one atomic each.
+// scan    : exclusive prefix sum of the bucket counts (chunk sums, then each
+//           chunk with the sum of those before it).
 // inverse : inv[offset[key] + rank] = i, the one scattered store per particle;
 // gather  : position j of the sorted copy (held in the workspace) takes
 //           element inv[j] of every array -- scattered reads, coalesced writes.
@@ -24,6 +24,7 @@ static size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 constexpr int kScanThreads = 512;
 constexpr int kScanItems = 8;
 constexpr int64_t kScanChunk = (int64_t)kScanThreads * kScanItems;
+constexpr int64_t kScanDirect = 8192;   // chunks whose sums each block adds up itself
 
 bool sort_plan(const gcb_particles *p, const gcb_grid *g, const gcb_params *prm, SortPlan &pl)
 {
@@ -89,59 +90,81 @@ static int caller_arrays(const gcb_particles *p, int ndim, void **a)
 
 struct KeyArgs {
     int64_t n;
-    int ndim, pair;
     const void *x[3];
-    const float *xlo[3];
     float inv_dx[3];
     int ncell[3], tile[3], ntile[3];
     int32_t *keys, *ranks, *hist;
     int frozen_key;
 };
 
-__global__ void k_sort_keys(const KeyArgs a)
+// Bound by the latency of a position's load and of its count's atomic, which
+// returns: four particles a thread keep four of each in flight.  Runs of equal
+// keys are found from the neighbouring lane; a match over the whole warp merges
+// a few more lanes but was what the kernel waited for.  FP32-pair positions:
+// the high parts alone decide the cell.  Measured (GB300): 2^24 particles 2D 235
+// -> 63 us, 3D 247 -> 89 us, 2^20 20 -> 7 us.
+constexpr int kKeyItems = 4;
+template <typename PosT, int ND>
+__global__ void __launch_bounds__(256) k_sort_keys(const KeyArgs a)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < a.n; base += stride) {
-        const int64_t i = base + threadIdx.x;
-        const bool v = i < a.n;
-        const unsigned act = __ballot_sync(0xffffffffu, v);
-        if (!v) continue;
-        int key = 0, mul = 1;
-        bool fin = true;
-        for (int d = 0; d < a.ndim; ++d) {
-            // the cell in FP32: a particle within rounding of a cell face may
-            // be filed in the neighbouring cell, which does not matter here
-            float xf;
-            if (a.pair) {
-                float lo = a.xlo[d][i];
-                xf = ((const float *)a.x[d])[i];
-                fin = fin && isfinite(xf) && isfinite(lo);
-            } else {
-                double xd = ((const double *)a.x[d])[i];
-                fin = fin && isfinite(xd);
-                xf = (float)xd;
-            }
-            float c = floorf(xf * a.inv_dx[d]);
-            int ci = fin ? (int)fminf(fmaxf(c, 0.0f), (float)(a.ncell[d] - 1)) : 0;
-            key += (ci / a.tile[d]) * mul;
-            mul *= a.ntile[d];
+    const int64_t stride = (int64_t)gridDim.x * 256 * kKeyItems;
+    for (int64_t base = (int64_t)blockIdx.x * 256 * kKeyItems; base < a.n; base += stride) {
+        int key[kKeyItems], head[kKeyItems], b[kKeyItems];
+        PosT x[kKeyItems][ND];
+#pragma unroll
+        for (int j = 0; j < kKeyItems; ++j) {
+            const int64_t i = base + j * 256 + threadIdx.x;
+#pragma unroll
+            for (int d = 0; d < ND; ++d)
+                x[j][d] = i < a.n ? static_cast<const PosT *>(a.x[d])[i] : PosT(0);
         }
-        if (!fin) key = a.frozen_key;
-        const unsigned peers = __match_any_sync(act, key);
-        const int leader = __ffs(peers) - 1;
-        const int before = __popc(peers & ((1u << lane) - 1u));
-        int b = 0;
-        if (lane == leader) b = atomicAdd(&a.hist[key], __popc(peers));
-        b = __shfl_sync(peers, b, leader);
-        a.keys[i] = key;
-        a.ranks[i] = b + before;
+#pragma unroll
+        for (int j = 0; j < kKeyItems; ++j) {
+            const bool v = base + j * 256 + threadIdx.x < a.n;
+            int k = 0, mul = 1;
+            bool fin = true;
+#pragma unroll
+            for (int d = 0; d < ND; ++d) {
+                // the cell in FP32: a particle within rounding of a cell face may
+                // be filed in the neighbouring cell, which does not matter here
+                fin = fin && isfinite(x[j][d]);
+                const float c = floorf((float)x[j][d] * a.inv_dx[d]);
+                const int ci = (int)fminf(fmaxf(c, 0.0f), (float)(a.ncell[d] - 1));
+                k += (a.tile[d] == 1 ? ci : ci / a.tile[d]) * mul;
+                mul *= a.ntile[d];
+            }
+            key[j] = v ? (fin ? k : a.frozen_key) : -1;
+            // runs: the lane where this lane's starts, and at a start its length
+            const int prev = __shfl_up_sync(0xffffffffu, key[j], 1);
+            const bool st = lane == 0 || key[j] != prev;
+            const unsigned m = __ballot_sync(0xffffffffu, st);
+            head[j] = 31 - __clz(m & (0xffffffffu >> (31 - lane)));
+            b[j] = 0;
+            if (st && v) {
+                const unsigned after = lane == 31 ? 0u : m >> (lane + 1);
+                const int len = after ? __ffs(after) : 32 - lane;
+                b[j] = atomicAdd(&a.hist[key[j]], len);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kKeyItems; ++j) {
+            const int r = __shfl_sync(0xffffffffu, b[j], head[j]) + lane - head[j];
+            const int64_t i = base + j * 256 + threadIdx.x;
+            if (i < a.n) {
+                a.keys[i] = key[j];
+                a.ranks[i] = r;
+            }
+        }
     }
 }
 
-// Exclusive scan of hist[0..m) in place, three passes: per-chunk sums,
-// a scan of the chunk sums (one block), and the per-chunk scan with its
-// offset.  Thread t of a block owns items [t*I, t*I + I) of the chunk.
+// Exclusive scan of hist[0..m) in place, two passes: per-chunk sums, and the
+// per-chunk scan from the sum of the chunks before it, which every block adds
+// up itself (16 KB of sums at the most 4096 + 1 chunks of a 256^3 grid, read
+// from L2; past kScanDirect chunks a single block scans the sums first).
+// Thread t of a block owns items [t*I, t*I + I) of the chunk, 16 bytes a load.
+// Measured (GB300): 256^3 cells 90 -> 40 us, 512x256 13.5 -> 6.4 us and a launch less.
 __device__ __forceinline__ int32_t block_excl_scan(int32_t v, int32_t *sh, int32_t &total)
 {
     const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
@@ -169,38 +192,71 @@ __device__ __forceinline__ int32_t block_excl_scan(int32_t v, int32_t *sh, int32
     return excl;
 }
 
+__device__ __forceinline__ void load_items(const int32_t *hist, int64_t base, int64_t m,
+                                           int32_t v[kScanItems])
+{
+    if (base + kScanItems <= m) {
+#pragma unroll
+        for (int k = 0; k < kScanItems; k += 4) {
+            const int4 q = *reinterpret_cast<const int4 *>(hist + base + k);
+            v[k] = q.x; v[k + 1] = q.y; v[k + 2] = q.z; v[k + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) v[k] = base + k < m ? hist[base + k] : 0;
+    }
+}
+
 __global__ void __launch_bounds__(kScanThreads) k_scan_sums(const int32_t *hist, int64_t m,
                                                             int32_t *bsum)
 {
     __shared__ int32_t sh[32];
-    const int64_t base = blockIdx.x * kScanChunk + (int64_t)threadIdx.x * kScanItems;
+    int32_t v[kScanItems];
+    load_items(hist, blockIdx.x * kScanChunk + (int64_t)threadIdx.x * kScanItems, m, v);
     int32_t s = 0;
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k)
-        if (base + k < m) s += hist[base + k];
+    for (int k = 0; k < kScanItems; ++k) s += v[k];
     int32_t tot;
     block_excl_scan(s, sh, tot);
     if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
 }
 
+// SUM: bsum holds the chunks' sums (else their exclusive scan)
+template <bool SUM>
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(int32_t *hist, int64_t m,
-                                                            const int32_t *boff)
+                                                            const int32_t *bsum)
 {
     __shared__ int32_t sh[32];
     const int64_t base = blockIdx.x * kScanChunk + (int64_t)threadIdx.x * kScanItems;
     int32_t v[kScanItems];
+    load_items(hist, base, m, v);
+    int32_t off = 0;
+    if constexpr (SUM) {
+        int32_t t = 0;
+        for (unsigned k = threadIdx.x; k < blockIdx.x; k += kScanThreads) t += bsum[k];
+        block_excl_scan(t, sh, off);
+    } else {
+        off = bsum[blockIdx.x];
+    }
     int32_t s = 0;
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        v[k] = base + k < m ? hist[base + k] : 0;
-        s += v[k];
-    }
+    for (int k = 0; k < kScanItems; ++k) s += v[k];
     int32_t tot;
-    int32_t run = block_excl_scan(s, sh, tot) + boff[blockIdx.x];
+    int32_t run = block_excl_scan(s, sh, tot) + off;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        if (base + k < m) hist[base + k] = run;
-        run += v[k];
+        const int32_t c = v[k];
+        v[k] = run;
+        run += c;
+    }
+    if (base + kScanItems <= m) {
+#pragma unroll
+        for (int k = 0; k < kScanItems; k += 4)
+            *reinterpret_cast<int4 *>(hist + base + k) = make_int4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k)
+            if (base + k < m) hist[base + k] = v[k];
     }
 }
 
@@ -344,11 +400,8 @@ gcb_status sort_into_workspace(const gcb_particles *p, const gcb_grid *g, const 
     }
     KeyArgs ka;
     ka.n = p->n;
-    ka.ndim = g->ndim;
-    ka.pair = p->pos_mode == GCB_POS_F32PAIR;
     for (int d = 0; d < 3; ++d) {
         ka.x[d] = p->x[d];
-        ka.xlo[d] = (const float *)p->x_lo[d];
         ka.inv_dx[d] = (float)(1.0 / g->dx[d]);
         ka.ncell[d] = (int)g->n[d];
         ka.tile[d] = pl.tile[d];
@@ -358,11 +411,23 @@ gcb_status sort_into_workspace(const gcb_particles *p, const gcb_grid *g, const 
     ka.ranks = ranks;
     ka.hist = hist;
     ka.frozen_key = (int)(pl.nbuckets - 1);
-    k_sort_keys<<<blocks_for(p->n, 256), 256, 0, st>>>(ka);
+    const int nk = blocks_for((p->n + kKeyItems - 1) / kKeyItems, 256);
+    if (p->pos_mode == GCB_POS_F32PAIR) {
+        if (g->ndim == 2) k_sort_keys<float, 2><<<nk, 256, 0, st>>>(ka);
+        else k_sort_keys<float, 3><<<nk, 256, 0, st>>>(ka);
+    } else {
+        if (g->ndim == 2) k_sort_keys<double, 2><<<nk, 256, 0, st>>>(ka);
+        else k_sort_keys<double, 3><<<nk, 256, 0, st>>>(ka);
+    }
     int32_t *bsum = (int32_t *)(ws + pl.off_bsum);
-    k_scan_sums<<<(unsigned)pl.nscan_blocks, kScanThreads, 0, st>>>(hist, pl.nbuckets, bsum);
-    k_scan<<<1, 1024, 0, st>>>(bsum, pl.nscan_blocks);
-    k_scan_down<<<(unsigned)pl.nscan_blocks, kScanThreads, 0, st>>>(hist, pl.nbuckets, bsum);
+    const unsigned nsc = (unsigned)pl.nscan_blocks;
+    k_scan_sums<<<nsc, kScanThreads, 0, st>>>(hist, pl.nbuckets, bsum);
+    if (pl.nscan_blocks <= kScanDirect) {
+        k_scan_down<true><<<nsc, kScanThreads, 0, st>>>(hist, pl.nbuckets, bsum);
+    } else {
+        k_scan<<<1, 1024, 0, st>>>(bsum, pl.nscan_blocks);
+        k_scan_down<false><<<nsc, kScanThreads, 0, st>>>(hist, pl.nbuckets, bsum);
+    }
     int32_t *inv = (int32_t *)(ws + pl.off_inv);
     k_inverse<<<blocks_for(p->n, 256), 256, 0, st>>>(p->n, keys, ranks, hist, inv);
     GatherArgs ga;
@@ -409,7 +474,8 @@ gcb_status sort_into_workspace(const gcb_particles *p, const gcb_grid *g, const 
     // (the 2D mixed state with FP32-pair positions: a step with a sort measured
     // 1.57 against 1.71 ms at 2^24 particles; the 3D one, 12 arrays, measured
     // slower than the generic gather, its registers halving the resident
-    // threads)
+    // threads, and three arrays at a time 551 against 531 us: what bounds it is
+    // the 32-byte sector read per scattered element)
     const int nb = blocks_for(p->n, 256);
     if (fixed && n4 == 9 && n8 == 0) k_gather_fixed<9, 0><<<nb, 256, 0, st>>>(fa);
     else k_gather_copy<<<nb, 256, 0, st>>>(ga);
