@@ -476,10 +476,16 @@ gcb_status gcb_push_ks(const gcb_particles *p, const gcb_grid_ks *gk, const gcb_
     if (!ws || !aligned(ws, 256)) { set_error("workspace NULL or not 256-byte aligned"); return GCB_EINVAL; }
     if (ws_bytes < kStatsBytes) { set_error("workspace too small"); return GCB_ENOMEM; }
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    unsigned long long *stats = (unsigned long long *)ws;
-    if (cudaMemsetAsync(stats, 0, kStatsBytes, st) != cudaSuccess) {
+    unsigned long long *stats = out ? (unsigned long long *)ws : nullptr;
+    if (stats && cudaMemsetAsync(stats, 0, kStatsBytes, st) != cudaSuccess) {
         set_error("cudaMemsetAsync: %s", cudaGetErrorString(cudaGetLastError()));
         return GCB_ECUDA;
+    }
+    if (stats && n_steps > 0) {   // the kernel without statistics readied too (see push_sr_impl)
+        gcb_particles none = *p;
+        none.n = 0;
+        s = push_step_ks(&none, &none, gk, kp, prm, st, nullptr);
+        if (s != GCB_OK) return s;
     }
     for (int step = 0; step < n_steps; ++step) {
         s = push_step_ks(p, p, gk, kp, prm, st, stats);
@@ -562,8 +568,8 @@ static gcb_status push_sr_impl(const gcb_particles *p, const gcb_grid *g, const 
     const bool fp64 = p->mom_dtype == GCB_F64;
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    unsigned long long *stats = (unsigned long long *)ws;
-    if (cudaMemsetAsync(stats, 0, kStatsBytes, st) != cudaSuccess) {
+    unsigned long long *stats = out || dst ? (unsigned long long *)ws : nullptr;
+    if (stats && cudaMemsetAsync(stats, 0, kStatsBytes, st) != cudaSuccess) {
         set_error("cudaMemsetAsync: %s", cudaGetErrorString(cudaGetLastError()));
         return GCB_ECUDA;
     }
@@ -588,15 +594,28 @@ static gcb_status push_sr_impl(const gcb_particles *p, const gcb_grid *g, const 
                 k = k < to_sort ? k : to_sort;
             }
         }
-        if (cur)
-            s = fp64 ? push_dep_step_f64(p, in, g, prm, cur, st, stats)
-                     : push_dep_step_f32(p, in, g, prm, cur, st, stats);
-        else if (prm->mirror == GCB_MIRROR_ON)
-            s = fp64 ? push_mir_step_f64(p, in, g, prm, st, stats)
-                     : push_mir_step_f32(p, in, g, prm, st, stats);
-        else
-            s = fp64 ? push_step_f64(p, in, g, prm, st, stats, k)
-                     : push_step_f32(p, in, g, prm, st, stats, k);
+        // a call with statistics also readies the kernel that a call without
+        // runs (an empty set: sized and loaded, not launched), so that a program
+        // that has pushed once may capture pushes into a graph
+        gcb_particles none = *p;
+        none.n = 0;
+        const bool ready = stats && step == 0;
+        if (cur) {
+            auto fn = fp64 ? (stats ? push_dep_step_f64 : push_dep_step_f64_quiet)
+                           : (stats ? push_dep_step_f32 : push_dep_step_f32_quiet);
+            if (ready) s = (fp64 ? push_dep_step_f64_quiet : push_dep_step_f32_quiet)(&none, &none, g, prm, cur, st, nullptr);
+            if (s == GCB_OK) s = fn(p, in, g, prm, cur, st, stats);
+        } else if (prm->mirror == GCB_MIRROR_ON) {
+            auto fn = fp64 ? (stats ? push_mir_step_f64 : push_mir_step_f64_quiet)
+                           : (stats ? push_mir_step_f32 : push_mir_step_f32_quiet);
+            if (ready) s = (fp64 ? push_mir_step_f64_quiet : push_mir_step_f32_quiet)(&none, &none, g, prm, st, nullptr);
+            if (s == GCB_OK) s = fn(p, in, g, prm, st, stats);
+        } else {
+            auto fn = fp64 ? (stats ? push_step_f64 : push_step_f64_quiet)
+                           : (stats ? push_step_f32 : push_step_f32_quiet);
+            if (ready) s = (fp64 ? push_step_f64_quiet : push_step_f32_quiet)(&none, &none, g, prm, st, nullptr, k);
+            if (s == GCB_OK) s = fn(p, in, g, prm, st, stats, k);
+        }
         if (s != GCB_OK) return s;
         step += k;
     }
@@ -854,16 +873,17 @@ gcb_status gcb_push_sr_ckpt(const gcb_particles *p, const gcb_grid *g, const gcb
     AdjLayout L;
     adj_layout(p, g, prm0, n_steps, ckpt_every, L);
     uint8_t *w = (uint8_t *)ws;
-    unsigned long long *stats = (unsigned long long *)ws;
-    if (cudaMemsetAsync(stats, 0, kStatsBytes, st) != cudaSuccess) {
+    unsigned long long *stats = out ? (unsigned long long *)ws : nullptr;
+    if (stats && cudaMemsetAsync(stats, 0, kStatsBytes, st) != cudaSuccess) {
         set_error("cudaMemsetAsync: %s", cudaGetErrorString(cudaGetLastError()));
         return GCB_ECUDA;
     }
     if (p->n > 0) {
         const bool fp64 = p->mom_dtype == GCB_F64;
         auto step = [&](const gcb_particles *in) {
-            return fp64 ? push_step_f64(p, in, g, &prm, st, stats)
-                        : push_step_adj_f32(p, in, g, &prm, st, stats);
+            if (fp64)
+                return (stats ? push_step_f64 : push_step_f64_quiet)(p, in, g, &prm, st, stats, 1);
+            return (stats ? push_step_adj_f32 : push_step_adj_f32_quiet)(p, in, g, &prm, st, stats);
         };
         for (int c = 0; c < L.nck; ++c) {
             const gcb_particles *in = p;
@@ -927,19 +947,17 @@ gcb_status gcb_adjoint_sr(const gcb_particles *p0, const gcb_grid *g, const gcb_
     adj_layout(p0, g, prm0, n_steps, ckpt_every, L);
     const size_t S = L.S;
     uint8_t *w = (uint8_t *)ws;
-    unsigned long long *stats = (unsigned long long *)w;
     uint8_t *ck = w + L.ck, *seg = w + L.seg, *tmp = w + L.tmp;
     const size_t nrec = (size_t)(g->n[0] * g->n[1] * g->n[2]) * 12;
-    if (cudaMemsetAsync(grad_rec, 0, nrec * sizeof(double), st) != cudaSuccess ||
-        cudaMemsetAsync(stats, 0, kStatsBytes, st) != cudaSuccess) {
+    if (cudaMemsetAsync(grad_rec, 0, nrec * sizeof(double), st) != cudaSuccess) {
         set_error("cudaMemsetAsync: %s", cudaGetErrorString(cudaGetLastError()));
         return GCB_ECUDA;
     }
     if (p0->n == 0) return GCB_OK;
     const bool fp64 = p0->mom_dtype == GCB_F64;
     auto step = [&](const gcb_particles *out, const gcb_particles *in) {
-        return fp64 ? push_step_f64(out, in, g, &prm, st, stats)
-                    : push_step_adj_f32(out, in, g, &prm, st, stats);
+        return fp64 ? push_step_f64_quiet(out, in, g, &prm, st, nullptr, 1)
+                    : push_step_adj_f32_quiet(out, in, g, &prm, st, nullptr);
     };
     gcb_particles tA = state_view(p0, nd, tmp), tB = state_view(p0, nd, tmp + S);
     if (!have_ckpt) {

@@ -25,28 +25,39 @@ void set_error(const char *fmt, ...);
 
 // One kernel pass over all particles, reading the arrays of `in` (the
 // caller's, or a sorted copy) and writing those of `p`; stats accumulate
-// into the device counters `stats` (ST_* layout).  nsteps > 1 takes that many
-// steps in the one launch (fused kernel).  Defined per precision.
-gcb_status push_step_f64(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
-                         const gcb_params *prm, cudaStream_t st, unsigned long long *stats,
-                         int nsteps = 1);
-gcb_status push_step_f32(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
-                         const gcb_params *prm, cudaStream_t st, unsigned long long *stats,
-                         int nsteps = 1);
-gcb_status push_step_adj_f32(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
-                             const gcb_params *prm, cudaStream_t st, unsigned long long *stats);
-// One unfused step with the mirror terms (push_mir_*.cu).
-gcb_status push_mir_step_f64(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
-                             const gcb_params *prm, cudaStream_t st, unsigned long long *stats);
-gcb_status push_mir_step_f32(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
-                             const gcb_params *prm, cudaStream_t st, unsigned long long *stats);
-// One unfused step that also adds the step's current to cur->J (push_dep_*.cu).
-gcb_status push_dep_step_f64(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
-                             const gcb_params *prm, const gcb_current *cur, cudaStream_t st,
-                             unsigned long long *stats);
-gcb_status push_dep_step_f32(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
-                             const gcb_params *prm, const gcb_current *cur, cudaStream_t st,
-                             unsigned long long *stats);
+// into the device counters `stats` (ST_* layout), or NULL: no statistics (the
+// _quiet forms below, their own kernels).  nsteps > 1 takes that many steps in
+// the one launch (fused kernel).  Defined per precision.
+#define GCB_PUSH_STEPS(SUFFIX)                                                                   \
+    gcb_status push_step_f64##SUFFIX(const gcb_particles *p, const gcb_particles *in,            \
+                                     const gcb_grid *g, const gcb_params *prm, cudaStream_t st,  \
+                                     unsigned long long *stats, int nsteps);                     \
+    gcb_status push_step_f32##SUFFIX(const gcb_particles *p, const gcb_particles *in,            \
+                                     const gcb_grid *g, const gcb_params *prm, cudaStream_t st,  \
+                                     unsigned long long *stats, int nsteps);                     \
+    /* one step of the adjoint's forward run */                                                  \
+    gcb_status push_step_adj_f32##SUFFIX(const gcb_particles *p, const gcb_particles *in,        \
+                                         const gcb_grid *g, const gcb_params *prm,               \
+                                         cudaStream_t st, unsigned long long *stats);            \
+    /* one unfused step with the mirror terms (push_mir_*.cu) */                                 \
+    gcb_status push_mir_step_f64##SUFFIX(const gcb_particles *p, const gcb_particles *in,        \
+                                         const gcb_grid *g, const gcb_params *prm,               \
+                                         cudaStream_t st, unsigned long long *stats);            \
+    gcb_status push_mir_step_f32##SUFFIX(const gcb_particles *p, const gcb_particles *in,        \
+                                         const gcb_grid *g, const gcb_params *prm,               \
+                                         cudaStream_t st, unsigned long long *stats);            \
+    /* one unfused step that also adds the step's current to cur->J (push_dep_*.cu) */           \
+    gcb_status push_dep_step_f64##SUFFIX(const gcb_particles *p, const gcb_particles *in,        \
+                                         const gcb_grid *g, const gcb_params *prm,               \
+                                         const gcb_current *cur, cudaStream_t st,                \
+                                         unsigned long long *stats);                             \
+    gcb_status push_dep_step_f32##SUFFIX(const gcb_particles *p, const gcb_particles *in,        \
+                                         const gcb_grid *g, const gcb_params *prm,               \
+                                         const gcb_current *cur, cudaStream_t st,                \
+                                         unsigned long long *stats);
+GCB_PUSH_STEPS()
+GCB_PUSH_STEPS(_quiet)
+#undef GCB_PUSH_STEPS
 
 // Adjoint (adjoint_sr.cu): one backward step for all particles whose
 // pre-step state is `s`; lam[7] (x0 x1 u0 u1 u2 dxp0 dxp1) is updated in

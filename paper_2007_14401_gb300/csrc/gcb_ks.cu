@@ -600,7 +600,8 @@ __device__ int ks_particle(const KsGrid<FT> &g, const StepCfg &c, double qm, int
 }
 
 // Three resident blocks per SM (at most 170 registers a thread).
-template <typename FT>
+// STATS: with the counters (a.stats), else none are kept.
+template <typename FT, bool STATS>
 __global__ void __launch_bounds__(TPB, 3) k_push_ks(const KsGrid<FT> g, const Args a)
 {
     __shared__ double s_x[3][TPB], s_u[3][TPB];
@@ -612,8 +613,8 @@ __global__ void __launch_bounds__(TPB, 3) k_push_ks(const KsGrid<FT> g, const Ar
     __shared__ unsigned long long s_acc[ST_COUNT];
     __shared__ double s_ek;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid < ST_COUNT) s_acc[tid] = 0ull;
-    if (tid == 0) s_ek = 0.0;
+    if (STATS && tid < ST_COUNT) s_acc[tid] = 0ull;
+    if (STATS && tid == 0) s_ek = 0.0;
     unsigned nb = 0, ng = 0, tg = 0, tb = 0, nc = 0, gf = 0, nf = 0, si = 0, mi = 0;
     unsigned ne = 0;   // frozen after leaving [r_in, r_out]
     double ek = 0.0;
@@ -738,10 +739,12 @@ __global__ void __launch_bounds__(TPB, 3) k_push_ks(const KsGrid<FT> g, const Ar
                 if (fail) ++gf;
                 si += it;
                 mi = max(mi, (unsigned)it);
-                double v[3];
-                raise(mfin, u, v);
-                const double u2 = dot(u, v);
-                ek = fma(u2, rcp64(1.0 + sqrt64(1.0 + u2)), ek);
+                if constexpr (STATS) {
+                    double v[3];
+                    raise(mfin, u, v);
+                    const double u2 = dot(u, v);
+                    ek = fma(u2, rcp64(1.0 + sqrt64(1.0 + u2)), ek);
+                }
             } else {
                 nfl |= GCB_FLAG_NONFINITE;
                 ++nf;
@@ -751,6 +754,7 @@ __global__ void __launch_bounds__(TPB, 3) k_push_ks(const KsGrid<FT> g, const Ar
             a.flags[gi] = nfl;
         }
     }
+    if constexpr (!STATS) return;
     unsigned vals[9] = {nb, ng, tg, tb, nc, gf, nf, si, mi};
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -807,7 +811,7 @@ __global__ void k_cell_size(int nr, int nth, double logr0, double dlogr, double 
     }
 }
 
-template <typename FT>
+template <typename FT, bool STATS>
 static gcb_status launch(const KsGrid<FT> &g, const Args &a, cudaStream_t st)
 {
     static int grid_cache[64] = {0};
@@ -819,7 +823,7 @@ static gcb_status launch(const KsGrid<FT> &g, const Args &a, cudaStream_t st)
     if (grid_cache[dev] == 0) {
         int nsm = 0, occ = 0;
         if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_push_ks<FT>, TPB, 0) != cudaSuccess) {
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_push_ks<FT, STATS>, TPB, 0) != cudaSuccess) {
             set_error("occupancy query failed");
             return GCB_ECUDA;
         }
@@ -828,7 +832,7 @@ static gcb_status launch(const KsGrid<FT> &g, const Args &a, cudaStream_t st)
     const int64_t ntiles = (a.np + TPB - 1) / TPB;
     if (ntiles == 0) return GCB_OK;
     const int nb = (int)(ntiles < grid_cache[dev] ? ntiles : grid_cache[dev]);
-    k_push_ks<FT><<<nb, TPB, 0, st>>>(g, a);
+    k_push_ks<FT, STATS><<<nb, TPB, 0, st>>>(g, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error("k_push_ks launch: %s", cudaGetErrorString(e));
@@ -877,7 +881,7 @@ static gcb_status push_step(const gcb_particles *p, const gcb_particles *in, con
     a.c.mu_mode = prm->mu_mode;
     a.c.basis = kp->kick_basis;
     a.stats = stats;
-    return launch<FT>(g, a, st);
+    return stats ? launch<FT, true>(g, a, st) : launch<FT, false>(g, a, st);
 }
 
 }  // namespace ks

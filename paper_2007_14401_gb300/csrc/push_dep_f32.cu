@@ -5,7 +5,7 @@
 
 namespace gcb {
 
-gcb_status push_dep_step_f32(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
+gcb_status GCB_FN(push_dep_step_f32)(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
                              const gcb_params *prm, const gcb_current *cur, cudaStream_t st,
                              unsigned long long *stats)
 {

@@ -5,7 +5,7 @@
 
 namespace gcb {
 
-gcb_status push_mir_step_f32(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
+gcb_status GCB_FN(push_mir_step_f32)(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
                              const gcb_params *prm, cudaStream_t st, unsigned long long *stats)
 {
     if (p->pos_mode == GCB_POS_F32PAIR)

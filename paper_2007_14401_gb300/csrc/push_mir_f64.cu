@@ -3,7 +3,7 @@
 
 namespace gcb {
 
-gcb_status push_mir_step_f64(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
+gcb_status GCB_FN(push_mir_step_f64)(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
                              const gcb_params *prm, cudaStream_t st, unsigned long long *stats)
 {
     return dispatch_push_mir<double, 0>(p, in, g, prm, st, stats);

@@ -380,8 +380,10 @@ __device__ __forceinline__ bool deposit_path(const PushArgs<R> &a, const int ib[
 // DEP (unfused only): each advanced particle-step also adds its current to a.J.
 // MIR (unfused only): the guiding-center step with the mirror terms.
 // GEN: gca_step_c where gca_lean.cuh would be used (the adjoint's forward run).
-template <typename R, int ND, int PM, int GM, bool FUSE, bool BT = false, bool DEP = false,
-          bool MIR = false, bool GEN = false>
+// STATS: with the counters (a.stats); without, the call did not ask for them
+// and neither the energy sum nor the counters' registers are spent on them.
+template <typename R, int ND, int PM, int GM, bool FUSE, bool BT, bool DEP, bool MIR, bool GEN,
+          bool STATS>
 __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP, BT>::n) k_push_sr(const PushArgs<R> a)
 {
     static_assert(!(DEP && FUSE), "deposition runs in unfused launches");
@@ -402,8 +404,8 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP, BT>:
     __shared__ unsigned long long s_acc[ST_COUNT];
     __shared__ double s_ek;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid < ST_COUNT) s_acc[tid] = 0ull;
-    if (tid == 0) s_ek = 0.0;
+    if (STATS && tid < ST_COUNT) s_acc[tid] = 0ull;
+    if (STATS && tid == 0) s_ek = 0.0;
 
     unsigned nb = 0, ng = 0, tg = 0, tb = 0, nc = 0, gf = 0, nf = 0, si = 0, mi = 0;
     unsigned nds = 0, npc = 0, nat = 0;   // DEP: skipped paths, pieces, atomics
@@ -714,8 +716,9 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP, BT>:
                 if (fail) ++gf;
                 si += it;
                 mi = max(mi, (unsigned)it);
-                R u2 = dot3(us, us) * sp.inv_c2;
-                if constexpr (sizeof(R) == 8) ek = fma(u2, rcp64(1.0 + sqrt64(1.0 + u2)), ek);
+                const R u2 = STATS ? dot3(us, us) * sp.inv_c2 : R(0);
+                if constexpr (!STATS) {}
+                else if constexpr (sizeof(R) == 8) ek = fma(u2, rcp64(1.0 + sqrt64(1.0 + u2)), ek);
                 else ek += (double)(u2 / (R(1) + sqrt(R(1) + u2)));
             } else {
                 // not advanced: the input state is kept (copied when the input
@@ -763,6 +766,7 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP, BT>:
       }
     }
 
+    if constexpr (!STATS) return;
     // block reduction of the counters
     unsigned vals[9] = {nb, ng, tg, tb, nc, gf, nf, si, mi};
 #pragma unroll
@@ -856,6 +860,13 @@ static void fill_args(PushArgs<R> &a, const gcb_particles *p, const gcb_particle
     a.stats = stats;
 }
 
+// Each translation unit of the push is compiled twice: with GCB_STATS 1, and as
+// its "quiet" form with 0 for the calls that do not ask for statistics.
+#ifndef GCB_STATS
+#define GCB_STATS 1
+#define GCB_FN(name) name
+#endif
+
 template <typename R, int ND, int PM, int GM, bool FUSE, bool BT = false, bool DEP = false,
           bool MIR = false, bool GEN = false>
 static gcb_status launch_push(const PushArgs<R> &a, cudaStream_t st)
@@ -870,7 +881,7 @@ static gcb_status launch_push(const PushArgs<R> &a, cudaStream_t st)
     if (grid == 0) {
         int nsm = 0, occ = 0;
         if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_push_sr<R, ND, PM, GM, FUSE, BT, DEP, MIR, GEN>,
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_push_sr<R, ND, PM, GM, FUSE, BT, DEP, MIR, GEN, GCB_STATS>,
                                                           Tile<R, ND>::n, 0) !=
                 cudaSuccess) {
             set_error("occupancy query failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -883,7 +894,7 @@ static gcb_status launch_push(const PushArgs<R> &a, cudaStream_t st)
     int64_t ntiles = (a.np + TPB - 1) / TPB;
     if (ntiles == 0) return GCB_OK;
     int nb = (int)(ntiles < grid ? ntiles : grid);
-    k_push_sr<R, ND, PM, GM, FUSE, BT, DEP, MIR, GEN><<<nb, TPB, 0, st>>>(a);
+    k_push_sr<R, ND, PM, GM, FUSE, BT, DEP, MIR, GEN, GCB_STATS><<<nb, TPB, 0, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error("kernel launch failed: %s", cudaGetErrorString(e));

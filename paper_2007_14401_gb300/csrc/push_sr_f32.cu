@@ -4,7 +4,7 @@
 
 namespace gcb {
 
-gcb_status push_step_f32(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
+gcb_status GCB_FN(push_step_f32)(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
                          const gcb_params *prm, cudaStream_t st, unsigned long long *stats,
                          int nsteps)
 {
@@ -27,7 +27,7 @@ static gcb_status step_adj(const gcb_particles *p, const gcb_particles *in, cons
     return launch_push<float, 2, PM, 2, false, false, false, false, true>(a, st);
 }
 
-gcb_status push_step_adj_f32(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
+gcb_status GCB_FN(push_step_adj_f32)(const gcb_particles *p, const gcb_particles *in, const gcb_grid *g,
                              const gcb_params *prm, cudaStream_t st, unsigned long long *stats)
 {
     return p->pos_mode == GCB_POS_F32PAIR ? step_adj<1>(p, in, g, prm, st, stats)
