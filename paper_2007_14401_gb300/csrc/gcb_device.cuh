@@ -95,9 +95,8 @@ __device__ __forceinline__ void cell_of<double>(const DevGrid<double> &g, int d,
                                                 double &t, int &i0, int &i1)
 {
     const int n = g.n[d];
-    const double s = l * g.inv_dx[d];
     int k;
-    t = s - floor64(s, n, k);
+    t = split64(l, g.inv_dx[d], n, k);
     int i = ib + k;
     i += i < 0 ? n : 0;
     i -= i >= n ? n : 0;
