@@ -77,11 +77,11 @@ WORKLOADS = {
                    grad_mode="grid", gca_tol=1e-7),
         # FMA-pipe busy fraction of this kernel in its ncu capture
         # (sm__pipe_fma_cycles_active, 2^21 particles; profiles/)
-        fma_pipe=0.288,
+        fma_pipe=0.294,
         # DRAM bytes (read + write) of one push launch at 2^24 particles, from
         # an ncu capture of this kernel (1 pass: dram__bytes_read.sum +
-        # dram__bytes_write.sum = 722.01 MB + 560.56 MB)
-        traffic_b=1282.57e6),
+        # dram__bytes_write.sum = 724.33 MB + 561.13 MB)
+        traffic_b=1285.46e6),
     "harris2d_fp64": dict(
         gen=_gen_harris, n=16384, precision="fp64", grid="f64", sort_every=0, tile=(1, 1),
         state_b=57, field_b=128 * 128 * 48, fp64_b=None,
@@ -100,7 +100,7 @@ WORKLOADS = {
         # particles) against the FP64 FMA rate measured live (libgcb_peak.so);
         # the derived peak 152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz = 1.2586
         # TFLOP/s is the fallback
-        alu=dict(flops=1724.4, peak=1.2586, peak_kind="fp64",
+        alu=dict(flops=1161.2, peak=1.2586, peak_kind="fp64",
                  peak_source="derived: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz "
                              "(ncu peak_sustained dfma 304 inst/clk)")),
     "sheet3d": dict(
@@ -110,7 +110,7 @@ WORKLOADS = {
              "power law in the sheet), |q/m| = 20",
         prec="mixed: FP32 fields and arithmetic, FP32-pair positions",
         extra=dict(grid=[256, 256, 256], dt=0.45, curvature=1, grad_mode="dw", gca_tol=1e-7),
-        fma_pipe=0.329),
+        fma_pipe=0.397),
     "sheet3d_literal": dict(
         gen=_gen_sheet3d_literal, n=1 << 26, precision="mixed", grid="f32", sort_every=8,
         tile=(1, 1, 1), state_b=49, field_b=256 ** 3 * 32, fp64_b=(73, 256 ** 3 * 48),
@@ -310,7 +310,7 @@ def pic_deposit(G, multi, ds, grid, p, sort_every, tile, ws, step, w, args, barr
            "vs_push_only": ms_push_max / ms_dep_max,
            "pieces_per_particle_step": cur.n_pieces / n, "atomics_per_particle_step": atom,
            "skipped": cur.n_skipped, "j_dtype": f,
-           "gpu_launches": K + 6 * n_sorts,
+           "gpu_launches": K + SORT_KERNELS * n_sorts,
            "method": "per step: J zeroed (torch), push with deposition (one kernel), J summed "
                      "over ranks; same sort schedule as the push-only block it is set against"}
     if dep_ms > 0 and rp.get(f):
@@ -520,16 +520,21 @@ def run_reference(args, rank, w):
     return 0
 
 
-def fused_launches(first, n_steps, fuse, sort_every):
+# Kernels of one sort on this file's grids: keys, two of the scan, inverse,
+# gather (past 2^25 buckets the scan has a third, 6 in all).
+SORT_KERNELS = 5
+
+
+def fused_launches(first, n_steps, fuse, sort_every, sort_kernels=6):
     """Kernels of n_steps fused steps: one push per launch (at most fuse steps,
-    none spanning a sort) plus the sort's 6 kernels at each sort step."""
+    none spanning a sort) plus the sort's kernels at each sort step."""
     count, j = 0, 0
     while j < n_steps:
         g = first + j
         k = min(fuse, n_steps - j)
         if sort_every > 0:
             if g % sort_every == 0:
-                count += 6
+                count += sort_kernels
             k = min(k, sort_every - g % sort_every)
         count += 1
         j += k
@@ -753,7 +758,7 @@ def main():
     barrier()
     clocks = clk.stop()
     ms = t0.elapsed_time(t1)
-    # steps that began with a sort run 6 more kernels; the push kernel's own
+    # steps that began with a sort run SORT_KERNELS more kernels; the push kernel's own
     # duration is taken from the steps without one
     first = args.warmup
     sorted_step = [sort_every > 0 and (first + k) % sort_every == 0 for k in range(args.steps)]
@@ -802,7 +807,8 @@ def main():
         tp_rate, tp_ms, _ = multi.whole_job_rate(n, fuse * kf, f0.elapsed_time(f1), device="cuda")
         tpm = {"value": tp_rate, "unit": METRIC, "fuse_steps": fuse, "steps": fuse * kf,
                "ms_per_step": tp_ms / (fuse * kf), "vs_pic_mode": tp_rate / value,
-               "gpu_launches": fused_launches(gpf.step_index, fuse * kf, fuse, sort_every),
+               "gpu_launches": fused_launches(gpf.step_index, fuse * kf, fuse, sort_every,
+                                              SORT_KERNELS),
                "note": "state kept on chip across the fused steps; bound by instruction "
                        "issue (the ALU side), not HBM"}
 
@@ -898,7 +904,7 @@ def main():
                                **({"kick_basis": args.ks_kick} if ks else {})),
                 "roofline": roofline,
                 "e2e": e2e,
-                "gpu_launches": args.steps + 6 * n_sorts,
+                "gpu_launches": args.steps + SORT_KERNELS * n_sorts,
                 "sort": {"every": sort_every, "sorts_in_timed_region": n_sorts,
                          "ms_step_with_sort": (sum(t for t, q in zip(step_ms, sorted_step) if q)
                                                / max(1, n_sorts)),
@@ -918,8 +924,8 @@ def main():
     return 0
 
 
-def adjoint_launches():
-    """Kernels of one forward + reverse sweep.  Forward: a sort (6 kernels)
+def adjoint_launches(sort_kernels=6):
+    """Kernels of one forward + reverse sweep.  Forward: a sort
     at each checkpoint, ADJ_STEPS pushes, then the composed order (one
     permutation per later checkpoint) and the scatter back to the caller's
     order.  Sweep: the composed order again and the gather of the adjoint
@@ -928,7 +934,7 @@ def adjoint_launches():
     projection."""
     nck = (ADJ_STEPS + ADJ_CKPT - 1) // ADJ_CKPT
     seg = [min(ADJ_CKPT, ADJ_STEPS - s * ADJ_CKPT) for s in range(nck)]
-    forward = 6 * nck + ADJ_STEPS + (nck - 1) + 1
+    forward = sort_kernels * nck + ADJ_STEPS + (nck - 1) + 1
     sweep = (nck - 1) + 1 + sum((L - 1) + L + 1 for L in seg) + 1
     return forward + sweep
 
@@ -1064,7 +1070,7 @@ def run_adjoint(args):
                             "dL_da_finite_modes": int(torch.isfinite(ga).sum()),
                             "dL_da_median_abs": float(ga[torch.isfinite(ga)].abs().median())
                             if bool(torch.isfinite(ga).any()) else None},
-                "gpu_launches": k * adjoint_launches(), "clocks": clocks, "e2e": None}
+                "gpu_launches": k * adjoint_launches(SORT_KERNELS), "clocks": clocks, "e2e": None}
         print(json.dumps(line), flush=True)
     if world > 1:
         dist.barrier()

@@ -16,7 +16,7 @@
 // bound by its pipe, 1343 -> 1019 pipe slots a particle-step of the 2D
 // reconnection push (2^20 particles 2.61 -> 1.95 ms a step; the 3D sheet,
 // 300007 particles, with gather_dw64 1.16 -> 0.79 ms); FP32 2D, bound by
-// issue, 1603 -> 1420 instructions (2^24 particles, 8 steps and a sort 9.83 ->
+// issue, 1603 -> 1401 instructions (2^24 particles, 8 steps and a sort 9.83 ->
 // 9.42 ms).  FP32 3D keeps gca_step_c and its record cache.
 #pragma once
 

@@ -585,8 +585,8 @@ __device__ __forceinline__ void bt_frame(const T E[3], const T B[3], T B2, T c, 
     om = T(1) - dot3(vE, vE) / (c * c);
 }
 
-// PROJ = false leaves out the projection of (b.grad)B and (v_E.grad)B onto
-// the plane normal to b: every use of (b.grad)b and (v_E.grad)b in the step
+// (b.grad)b and (v_E.grad)b are left without the projection of (b.grad)B and
+// (v_E.grad)B onto the plane normal to b: every use of (b.grad)b and (v_E.grad)b in the step
 // is b x (.) or v_E . (.), which annihilates the component along b (v_E is
 // normal to B), so the step's results are the same up to rounding.
 // BT = true builds the exact frame (bt_frame) in place of the simplified
@@ -594,7 +594,7 @@ __device__ __forceinline__ void bt_frame(const T E[3], const T B[3], T B2, T c, 
 // are (b*.grad)b and (v_E.grad)b with grad b that of the lab-frame b = B/B
 // (projected), the records carrying no grad E.
 // MIR = true also forms grad |B|: d_i |B| = b_j d_i B_j (the mirror terms).
-template <typename R, int ND, bool GRADS, bool PROJ = true, bool BT = false, bool MIR = false>
+template <typename R, int ND, bool GRADS, bool BT = false, bool MIR = false>
 __device__ __forceinline__ void make_frame(const FieldPt<R, ND> &F, R c, R inv_c2, Frame<R> &f)
 {
     if constexpr (BT) {
@@ -645,9 +645,8 @@ __device__ __forceinline__ void make_frame(const FieldPt<R, ND> &F, R c, R inv_c
     R B2 = dot3(F.B, F.B);
     f.ok = B2 > R(0);
     if (!f.ok) B2 = R(1);
-    R ib = PROJ ? R(1) / sqrt(B2) : inv_sqrt(B2);
-    f.Bmag = PROJ ? sqrt(B2) : B2 * ib;
-    if (PROJ) ib = R(1) / f.Bmag;
+    R ib = inv_sqrt(B2);
+    f.Bmag = B2 * ib;
     f.ib = ib;
     R ib2 = ib * ib;
 #pragma unroll
@@ -659,7 +658,7 @@ __device__ __forceinline__ void make_frame(const FieldPt<R, ND> &F, R c, R inv_c
     R beta2 = dot3(f.vE, f.vE) * inv_c2;
     R om = one_minus_beta2<R>(F.E, F.B, B2, c, beta2);
     f.ok = f.ok && (om > R(0));
-    f.kappa = PROJ ? R(1) / sqrt(f.ok ? om : R(1)) : inv_sqrt(f.ok ? om : R(1));
+    f.kappa = inv_sqrt(f.ok ? om : R(1));
     f.Epar = dot3(F.E, f.b);
     if (GRADS) {
         // w = (b.grad)B, y = (v_E.grad)B; then (b.grad)b = (w - b (b.w))/B etc.
@@ -675,19 +674,10 @@ __device__ __forceinline__ void make_frame(const FieldPt<R, ND> &F, R c, R inv_c
             w[j] = sw;
             y[j] = sy;
         }
-        if (PROJ) {
-            R bw = dot3(f.b, w), by = dot3(f.b, y);
 #pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                f.bgb[j] = fma(-f.b[j], bw, w[j]) * ib;
-                f.vgb[j] = fma(-f.b[j], by, y[j]) * ib;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                f.bgb[j] = w[j] * ib;
-                f.vgb[j] = y[j] * ib;
-            }
+        for (int j = 0; j < 3; ++j) {
+            f.bgb[j] = w[j] * ib;
+            f.vgb[j] = y[j] * ib;
         }
         if constexpr (MIR) {
 #pragma unroll
@@ -722,38 +712,9 @@ __device__ __forceinline__ R gamma_gc(const Frame<R> &f, const StepPar<R> &s, R 
     return f.kappa * sqrt(R(1) + fma(upar, upar, perp2(f, s, mu, uperp)) * s.inv_c2);
 }
 
-// Eq. (curvdrift): v_c = (m c kappa^2/(q B)) b x [(u_par^2/Gamma)(b.grad)b + u_par (v_E.grad)b].
-template <typename R>
-__device__ __forceinline__ void vcurv(const Frame<R> &f, const StepPar<R> &s, R upar, R G, R vc[3])
-{
-    if (!s.curvature) { vc[0] = vc[1] = vc[2] = R(0); return; }
-    R a[3];
-    R k2 = upar * upar / G;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) a[k] = fma(k2, f.bgb[k], upar * f.vgb[k]);
-    R x[3];
-    cross3(f.b, a, x);
-    R pref = s.c * f.kappa * f.kappa / (s.qm * f.Bmag);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) vc[k] = pref * x[k];
-}
-
-// Guiding-center velocity, Eq. (dRdt): u_par b / Gamma + v_E + v_c.
-template <typename R>
-__device__ __forceinline__ void gc_vel(const Frame<R> &f, const StepPar<R> &s, R upar, R mu, R uperp,
-                                       R V[3])
-{
-    R G = gamma_gc(f, s, upar, mu, uperp);
-    R vc[3];
-    vcurv(f, s, upar, G, vc);
-    R ig = upar / G;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) V[k] = fma(ig, f.b[k], f.vE[k] + vc[k]);
-}
-
-// The same two quantities from 1/Gamma and cq = c/(q/m), as the push
-// evaluates them: v_c with prefactor cq kappa^2/B, and u_par b/Gamma + v_E +
-// v_c with the one reciprocal of Gamma.
+// Eq. (curvdrift), v_c = (m c kappa^2/(q B)) b x [(u_par^2/Gamma)(b.grad)b +
+// u_par (v_E.grad)b], and the guiding-center velocity, Eq. (dRdt), u_par
+// b/Gamma + v_E + v_c, from the one reciprocal 1/Gamma and cq = c/(q/m).
 template <typename R>
 __device__ __forceinline__ void vcurv_ig(const Frame<R> &f, const StepPar<R> &s, R cq, R upar, R iG,
                                          R vc[3])
@@ -899,14 +860,14 @@ __device__ __forceinline__ bool gca_step_c(const Gth &gth, const StepPar<R> &s, 
     const R cq = s.c / s.qm;
     FieldPt<R, ND> F;
     Frame<R> f0, f;
-    make_frame<R, ND, GR, false, BT, MIR>(F0, s.c, s.inv_c2, f0);
+    make_frame<R, ND, GR, BT, MIR>(F0, s.c, s.inv_c2, f0);
 
     // conversion at R^{n-1/2} = x^n - dxp/2 (Sec. 3.1)
     R pt[ND];
 #pragma unroll
     for (int d = 0; d < ND; ++d) pt[d] = fma(R(-0.5), dxp[d], ln[d]);
     gat(pt, F);
-    make_frame<R, ND, GR, false, BT>(F, s.c, s.inv_c2, f);
+    make_frame<R, ND, GR, BT>(F, s.c, s.inv_c2, f);
     if (!(f0.ok && f.ok)) return false;
     R Gfull = sqrt(R(1) + dot3(u, u) * s.inv_c2);
     R upar = dot3(u, f.b);
@@ -990,7 +951,7 @@ __device__ __forceinline__ bool gca_step_c(const Gth &gth, const StepPar<R> &s, 
 #pragma unroll
         for (int d = 0; d < ND; ++d) pt[d] = ln[d] + dk[d];
         gat(pt, F);
-        make_frame<R, ND, GR, false, BT, MIR>(F, s.c, s.inv_c2, f);
+        make_frame<R, ND, GR, BT, MIR>(F, s.c, s.inv_c2, f);
         okall = okall && f.ok;   // a bad frame fails the step after the loop
         gc_vel_ig<R, MIR>(f, s, cq, upn, mu, uperp, V);
     }
@@ -1000,7 +961,7 @@ __device__ __forceinline__ bool gca_step_c(const Gth &gth, const StepPar<R> &s, 
 #pragma unroll
     for (int d = 0; d < ND; ++d) pt[d] = fma(R(0.5), dk[d], ln[d]);
     gat(pt, F);
-    make_frame<R, ND, GR, false, BT>(F, s.c, s.inv_c2, f);
+    make_frame<R, ND, GR, BT>(F, s.c, s.inv_c2, f);
     if (!f.ok) return false;
     R Gp = gamma_gc(f, s, upn, mu, uperp);
     vcurv_ig(f, s, cq, upn, R(1) / Gp, vc);

@@ -25,7 +25,7 @@ constexpr int NWARP = TPB / 32;
 // helpers of real64.cuh, closed forms that share their factors, and in the
 // guiding-center iterations the metric's derivative along b only.  Measured
 // (GB300, 2^20 particles, FP32 records, local-frame kicks): 1391 -> 1017 pipe
-// slots a particle-step, 3.17 -> 2.32 ms; 100003 particles, FP64 records,
+// slots a particle-step, 3.17 -> 2.32 ms (2.27 without counters); 100003 particles, FP64 records,
 // global-basis kicks: 382 -> 285 us.
 
 // Kerr-Schild 3+1 quantities (M = 1) at a point:

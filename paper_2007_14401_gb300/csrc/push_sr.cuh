@@ -41,10 +41,12 @@ struct Tile {
 #define GCB_UNIFORM_TILES 1
 #endif
 // minimum resident threads per SM requested from the register allocator:
-// FP32 2D 576 (at most 112 registers a thread; 8 steps of 2^24 particles and
-// their sort 8.32 ms at 512, 7.62 at 576, 7.60 at 640, 7.76 at 704, 8.25 at 768;
-// 2^22 with deposition 2.82, 2.68, 2.71, 2.81, 2.96 ms), and 512 in the exact
-// frame, whose longer frame spills 240 B at 112; FP32 3D 384 (at most
+// FP32 2D 576 (with the four partitions' rounding 96 registers a thread, no
+// more than 16 B spilled and 20 resident warps; 8 steps of 2^24 particles and
+// their sort 8.32 ms at 512, 7.62 at 576, 7.60 at 640, 7.76 at 704, 8.25 at
+// 768; 2^22 with deposition 2.82, 2.68, 2.71, 2.81, 2.96 ms; without counters
+// 576, 640 and 704 within 1% of one another), and 512 in the exact frame,
+// whose longer frame (116 registers) spills 108 B at 96; FP32 3D 384 (at most
 // 170 registers: 184 unconstrained leaves 256 threads, which measured 16%
 // slower, and 512 spills)
 #ifndef GCB_MIN_THREADS_F32_2D
