@@ -106,6 +106,24 @@ __device__ __forceinline__ void cell_of<double>(const DevGrid<double> &g, int d,
     i1 = j;
 }
 
+// The weights of a cell's nodes in FP64, each pair's second by difference from
+// the pair's sum: 5 operations in 2D, 13 in 3D (products of 1D weights: 6, 19).
+template <int ND>
+__device__ __forceinline__ void weights64(const double t[ND], double W[1 << ND])
+{
+    W[3] = t[0] * t[1];
+    W[1] = t[0] - W[3];
+    W[2] = t[1] - W[3];
+    W[0] = (1.0 - t[0]) - W[2];
+    if constexpr (ND == 3) {
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            W[o + 4] = W[o] * t[2];
+            W[o] -= W[o + 4];
+        }
+    }
+}
+
 // Linear-shape-function gather (Sec. 4 intro): F(x) = sum_N F_N W(x - x_N),
 // grad F(x) = sum_N F_N grad W(x - x_N), W the product of 1D hat functions.
 // GM = 0: E and B only;  1: gradients of B from grad W (differentiate the
@@ -132,6 +150,9 @@ __device__ __forceinline__ void gather(const DevGrid<R> &g, const int ib[ND], co
     // elements needed from each record
     constexpr int NEED = (GM == 2) ? 6 + 3 * ND : 6;
     constexpr int NCHUNK = (NEED + CH - 1) / CH;
+    constexpr bool DIFF = sizeof(R) == 8 && GM != 1;   // weights by difference
+    R Wd[NC];
+    if constexpr (DIFF) weights64<ND>(t, Wd);
 #pragma unroll
     for (int o = 0; o < NC; ++o) {
         int node;
@@ -151,6 +172,7 @@ __device__ __forceinline__ void gather(const DevGrid<R> &g, const int ib[ND], co
         R W = w[0];
 #pragma unroll
         for (int d = 1; d < ND; ++d) W *= w[d];
+        if constexpr (DIFF) W = Wd[o];
         R v[NCHUNK * CH];
         const R *rp = g.rec + (size_t)node * g.stride;
 #pragma unroll
@@ -417,7 +439,9 @@ struct RawGrad { static constexpr bool value = sizeof(R) == 8 && GM == 1; };
 // along one axis after the other: the differences that a field component's
 // interpolation takes are also its gradient (22 FP64 operations a component in
 // 3D, 8 in 2D, where weights and their derivatives take 32 and 12, and their
-// products 60 and 12 more a gather).  F.dB is left per cell (RawGrad).
+// products 60 and 12 more a gather).  E in 3D, of which no gradient is taken,
+// is summed with the weights instead (37 operations a gather for 42; 8 steps of
+// 3e5 particles 6.06 -> 5.87 ms).  F.dB is left per cell (RawGrad).
 template <int ND>
 __device__ __forceinline__ void gather_dw64(const DevGrid<double> &g, const int ib[ND],
                                             const double l[ND], FieldPt<double, ND> &F)
@@ -434,6 +458,8 @@ __device__ __forceinline__ void gather_dw64(const DevGrid<double> &g, const int 
         if (ND == 3) node += ((o & 4) ? i1[ND - 1] : i0[ND - 1]) * g.n[1] * g.n[0];
         rp[o] = g.rec + (size_t)node * g.stride;
     }
+    double W[NC];
+    if constexpr (ND == 3) weights64<ND>(t, W);
 #pragma unroll
     for (int q = 0; q < 3; ++q) {          // components 2q and 2q + 1 of (E, B)
         double v[NC][2];
@@ -442,6 +468,14 @@ __device__ __forceinline__ void gather_dw64(const DevGrid<double> &g, const int 
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int c = 2 * q + h;
+            if constexpr (ND == 3) {
+                if (c < 3) {
+                    F.E[c] = W[0] * v[0][h];
+#pragma unroll
+                    for (int o = 1; o < NC; ++o) F.E[c] = fma(W[o], v[o][h], F.E[c]);
+                    continue;
+                }
+            }
             double d[NC / 2], w[NC / 2];   // along x: differences and values
 #pragma unroll
             for (int o = 0; o < NC / 2; ++o) {
