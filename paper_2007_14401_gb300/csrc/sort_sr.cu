@@ -352,7 +352,7 @@ __global__ void k_gather_fixed(const GatherFixedArgs a)
 }
 
 // Element-wise permutation of up to 16 arrays: dst[j] = src[idx[j]]
-// (gather) or dst[idx[j]] = src[j] (scatter).
+// (gather) or dst[idx[j]] = src[j] (scatter); a copy where idx is NULL.
 struct PermArgs {
     int64_t n;
     int na;
@@ -367,7 +367,7 @@ __global__ void k_permute(const PermArgs a)
 {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < a.n;
          j += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = a.idx[j];
+        const int64_t i = a.idx ? a.idx[j] : j;
         const int64_t from = a.scatter ? j : i, to = a.scatter ? i : j;
 #pragma unroll 1
         for (int k = 0; k < a.na; ++k) {
@@ -388,7 +388,8 @@ static int blocks_for(int64_t n, int tpb)
 }
 
 gcb_status sort_into_workspace(const gcb_particles *p, const gcb_grid *g, const SortPlan &pl,
-                               cudaStream_t st, uint8_t *ws, SortedView &out)
+                               cudaStream_t st, uint8_t *ws, SortedView &out,
+                               const gcb_particles *into)
 {
     if (p->n == 0) return GCB_OK;
     int32_t *keys = (int32_t *)(ws + pl.off_keys);
@@ -433,10 +434,12 @@ gcb_status sort_into_workspace(const gcb_particles *p, const gcb_grid *g, const 
     GatherArgs ga;
     ga.n = p->n;
     void *src[14];
+    void *own[14] = {};
     ga.na = caller_arrays(p, g->ndim, src);
+    if (into) caller_arrays(into, g->ndim, own);
     for (int k = 0; k < ga.na; ++k) {
         ga.src[k] = src[k];
-        ga.dst[k] = src[k] ? (void *)(ws + pl.off_arr[k]) : nullptr;
+        ga.dst[k] = !src[k] ? nullptr : (own[k] ? own[k] : (void *)(ws + pl.off_arr[k]));
         ga.es[k] = pl.es[k];
         out.arr[k] = ga.dst[k];
     }
