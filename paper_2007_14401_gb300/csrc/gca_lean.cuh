@@ -33,8 +33,17 @@ __device__ __forceinline__ bool pos_finite(double x) { return !not_pos_normal(x)
 
 // Local frame at a point: v_E, and through B2 = |B|^2, ib = 1/|B|, om = 1 -
 // v_E^2/c^2 and kap = 1/sqrt(om) the factors of the drift terms.
+// The unit of the fields is the caller's.  FP64's exponents hold |E x B|^2 and
+// |B|^-3 for |B| of 1e-77 to 1e77, so that the factors 1/|B| are gathered into
+// one; FP32's hold |E x B|^2 for 1e-9 to 4e9 only.  There (F32) |v_E|^2 is taken
+// from v_E and every product of two fields meets its 1/|B| before the next
+// (lean_drift, the u_par update), which keeps all of them within |B|^2, good for
+// 1e-19 to 1e19 (from 1e-19 sqrt(c) up, c/|B|^2 being one of them).  It costs nothing worth having (GB300, 2^24 particles in 2D, 8
+// steps and their sort: one factor |B|^-3 8.18 ms, this 8.21; the order of
+// lean_drift's prefactor decides, with kappa^2 apart 8 B more spilled, 8.37).
 template <typename R>
 struct LeanFrame {
+    static constexpr bool F32 = sizeof(R) == 4;
     R B2, ib, ib2, om, kap, vE[3];
     bool ok;
     __device__ __forceinline__ R Bk() const { return B2 * ib * kap; }      // |B| kappa
@@ -48,21 +57,25 @@ struct LeanFrame {
 };
 
 template <typename R, int ND>
-__device__ __forceinline__ void lean_frame(const FieldPt<R, ND> &F, R c, LeanFrame<R> &f)
+__device__ __forceinline__ void lean_frame(const FieldPt<R, ND> &F, const StepPar<R> &s,
+                                           LeanFrame<R> &f)
 {
     f.B2 = dot3(F.B, F.B);
     f.ib = rsq(f.B2);
     f.ib2 = f.ib * f.ib;
     R x[3];
     cross3(F.E, F.B, x);
-    const R v2 = dot3(x, x) * f.ib2;       // |E x B|^2/B^2 = B^2 v_E^2/c^2
-    if constexpr (sizeof(R) == 8) f.om = fma(-v2, f.ib2, R(1));
-    else f.om = one_minus_beta2<R>(F.E, F.B, f.B2, c, v2 * f.ib2);
-    f.ok = pos_finite(f.B2) && pos_finite(f.om);
-    f.kap = rsq(f.om);
-    const R cv = c * f.ib2;
+    const R cv = s.c * f.ib2;
 #pragma unroll
     for (int k = 0; k < 3; ++k) f.vE[k] = cv * x[k];
+    if constexpr (LeanFrame<R>::F32) {
+        f.om = one_minus_beta2<R>(F.E, F.B, f.B2, s.c, dot3(f.vE, f.vE) * s.inv_c2);
+    } else {
+        const R v2 = dot3(x, x) * f.ib2;   // |E x B|^2/B^2 = B^2 v_E^2/c^2
+        f.om = fma(-v2, f.ib2, R(1));
+    }
+    f.ok = pos_finite(f.B2) && pos_finite(f.om);
+    f.kap = rsq(f.om);
 }
 
 // Drift velocity v_E + v_c (+ grad-B drift) for upar and iG = 1/Gamma, and
@@ -74,6 +87,7 @@ __device__ __forceinline__ void lean_drift(const FieldPt<R, ND> &F, const LeanFr
                                            const StepPar<R> &s, const R gs[ND], R upar, R iG, R mu2,
                                            R &ig, R v[3])
 {
+    constexpr bool F32 = LeanFrame<R>::F32;
     ig = upar * (iG * f.ib);
     if (s.curvature) {
         R a[3], x[3];
@@ -81,11 +95,14 @@ __device__ __forceinline__ void lean_drift(const FieldPt<R, ND> &F, const LeanFr
         for (int i = 0; i < ND; ++i) {
             R gi = fma(ig, F.B[i], f.vE[i]);
             if (RAW) gi *= gs[i];
+            if (F32) gi *= f.ib;
 #pragma unroll
             for (int j = 0; j < 3; ++j) a[j] = i == 0 ? gi * F.dB[i][j] : fma(gi, F.dB[i][j], a[j]);
         }
         cross3(F.B, a, x);
-        const R pf = (s.cq * upar) * (f.ib * f.ib2) * (f.kap * f.kap);
+        R pf = s.cq * upar;               // c kappa^2 u_par/(q |B|^3); F32: |B|^2
+        if constexpr (F32) pf = pf * (f.ib * f.kap) * (f.ib * f.kap);
+        else pf = pf * (f.ib * f.ib2) * (f.kap * f.kap);
 #pragma unroll
         for (int k = 0; k < 3; ++k) v[k] = fma(pf, x[k], f.vE[k]);
     } else {
@@ -95,9 +112,14 @@ __device__ __forceinline__ void lean_drift(const FieldPt<R, ND> &F, const LeanFr
     if constexpr (MIR) {
         R h[3] = {R(0), R(0), R(0)}, x[3];
 #pragma unroll
-        for (int i = 0; i < ND; ++i) h[i] = RAW ? dot3(F.B, F.dB[i]) * gs[i] : dot3(F.B, F.dB[i]);
+        for (int i = 0; i < ND; ++i) {    // |B| grad|B|; F32: grad|B|
+            h[i] = dot3(F.B, F.dB[i]);
+            if (RAW) h[i] *= gs[i];
+            if (F32) h[i] *= f.ib;
+        }
         cross3(F.B, h, x);
-        const R pg = R(0.5) * s.cq * f.kap * mu2 * iG * f.ib2 * f.ib;
+        R pg = R(0.5) * s.cq * f.kap * mu2 * iG * f.ib2;
+        if (!F32) pg *= f.ib;
 #pragma unroll
         for (int k = 0; k < 3; ++k) v[k] = fma(pg, x[k], v[k]);
     }
@@ -129,13 +151,13 @@ __device__ __forceinline__ bool gca_step_lean(const Gth &gth, const StepPar<R> &
                                               int &iters, bool &nonconv,
                                               R *vz = nullptr)
 {
-    constexpr bool RAW = RawGrad<R, GM>::value;
+    constexpr bool RAW = RawGrad<R, GM>::value, F32 = LeanFrame<R>::F32;
     R gs[ND];
 #pragma unroll
     for (int d = 0; d < ND; ++d) gs[d] = gth.g.inv_dx[d];
     FieldPt<R, ND> F;
     LeanFrame<R> f0, f;
-    lean_frame<R, ND>(F0, s.c, f0);
+    lean_frame<R, ND>(F0, s, f0);
 
     // conversion at R^{n-1/2} = x^n - dxp/2 (Sec. 3.1): u = u_par b + (v_E +
     // v_c) Gamma + u_g
@@ -143,7 +165,7 @@ __device__ __forceinline__ bool gca_step_lean(const Gth &gth, const StepPar<R> &
 #pragma unroll
     for (int d = 0; d < ND; ++d) pt[d] = fma(R(-0.5), dxp[d], ln[d]);
     gth(ib, pt, F);
-    lean_frame<R, ND>(F, s.c, f);
+    lean_frame<R, ND>(F, s, f);
     if (!(f0.ok && f.ok)) return false;
     R v[3], ig;
     R G = fma(dot3(u, u), s.inv_c2, R(1));
@@ -166,14 +188,14 @@ __device__ __forceinline__ bool gca_step_lean(const Gth &gth, const StepPar<R> &
     R upn;
     const R P0 = s.mu_mode ? up2 : mu2 * f0.Bk();
     if constexpr (MIR) {
-        R bg = R(0);                      // B . grad|B| |B|
+        R bg = R(0);                      // B . grad|B| |B|; F32: B . grad|B|
 #pragma unroll
         for (int i = 0; i < ND; ++i) {
-            const R h = F0.B[i] * dot3(F0.B, F0.dB[i]);
+            const R h = F0.B[i] * (F32 ? f0.ib * dot3(F0.B, F0.dB[i]) : dot3(F0.B, F0.dB[i]));
             bg += RAW ? h * gs[i] : h;
         }
         const R iG0 = rsq(fma(fma(upar, upar, P0), s.inv_c2, R(1))) * (f0.om * f0.kap);
-        fm = R(-0.5) * s.dt * mu2 * bg * f0.ib2 * iG0 * (f0.om * f0.kap);
+        fm = R(-0.5) * s.dt * mu2 * bg * (F32 ? f0.ib : f0.ib2) * iG0 * (f0.om * f0.kap);
     }
     if (!s.curvature) {
         upn = fma(s.qm * s.dt, Epar, upar) + fm;
@@ -183,11 +205,12 @@ __device__ __forceinline__ bool gca_step_lean(const Gth &gth, const StepPar<R> &
         for (int i = 0; i < ND; ++i) {
             R z = dot3(f0.vE, F0.dB[i]);
             if (RAW) z *= gs[i];
+            if (F32) z *= f0.ib;
             a = i == 0 ? F0.B[i] * z : fma(F0.B[i], z, a);
             gg = i == 0 ? f0.vE[i] * z : fma(f0.vE[i], z, gg);
         }
-        a *= f0.ib2;
-        gg *= f0.ib;
+        a *= F32 ? f0.ib : f0.ib2;
+        if (!F32) gg *= f0.ib;
         const R ha = s.half_dt * a;
         const R hg = s.half_dt * gg;
         const R D = R(1) - ha;
@@ -275,7 +298,7 @@ __device__ __forceinline__ bool gca_step_lean(const Gth &gth, const StepPar<R> &
 #pragma unroll
         for (int d = 0; d < ND; ++d) pt[d] = ln[d] + dk[d];
         gth(ib, pt, F);
-        lean_frame<R, ND>(F, s.c, f);
+        lean_frame<R, ND>(F, s, f);
         okall = okall && f.ok;   // a bad frame fails the step after the loop
         velocity(F, f, V);
     }
@@ -285,7 +308,7 @@ __device__ __forceinline__ bool gca_step_lean(const Gth &gth, const StepPar<R> &
 #pragma unroll
     for (int d = 0; d < ND; ++d) pt[d] = fma(R(0.5), dk[d], ln[d]);
     gth(ib, pt, F);
-    lean_frame<R, ND>(F, s.c, f);
+    lean_frame<R, ND>(F, s, f);
     if (!f.ok) return false;
     R Gp = gam2(f);
     const R rg = rsq(Gp);
