@@ -26,12 +26,14 @@ __device__ __forceinline__ double rcp_r(double x) { return rcp64(x); }
 // v_E^2/c^2, 1/kappa and the unscaled directional derivatives w = (b.grad)B, y =
 // (v_E.grad)B kept.  bgb = w/|B| and vgb = y/|B| are left unprojected: every
 // use is b x (.) or v_E . (.), which annihilates their component along b for
-// any fields, so that the step's derivative does not depend on it.
+// any fields, so that the step's derivative does not depend on it.  1 -
+// v_E^2/c^2 from v_E, as the forward step's frame has it: |E x B|^2 is a fourth
+// power of the field, which FP32 holds for 1e-9 < |B| < 4e9 only.
 template <typename T, int ND>
 struct RFrame {
     T Bmag, ib, ib2, b[3], x[3], vE[3], om, kappa, ikap, Epar, w[3], y[3], bgb[3], vgb[3];
 
-    __device__ __forceinline__ void make(const FieldPt<T, ND> &F, T c)
+    __device__ __forceinline__ void make(const FieldPt<T, ND> &F, T c, T inv_c2)
     {
         const T B2 = dot3(F.B, F.B);
         ib = rsq_r(B2);
@@ -41,7 +43,7 @@ struct RFrame {
         const T cv = c * ib2;
 #pragma unroll
         for (int k = 0; k < 3; ++k) { b[k] = F.B[k] * ib; vE[k] = cv * x[k]; }
-        om = one_minus_beta2<T>(F.E, F.B, B2, c, dot3(x, x) * (ib2 * ib2));
+        om = one_minus_beta2<T>(F.E, F.B, B2, c, dot3(vE, vE) * inv_c2);
         kappa = rsq_r(om);
         ikap = om * kappa;
         Epar = dot3(F.E, b);

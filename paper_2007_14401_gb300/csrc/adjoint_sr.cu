@@ -549,12 +549,12 @@ __device__ __forceinline__ void gather_bwd(const DevGrid<T> &g, NodeCache<T> &nc
 // field and frame at gather point `pt` (FCache numbering) located at p
 template <typename T>
 __device__ __forceinline__ void frame_at(const DevGrid<T> &g, const FCache<T> &fc, int pt,
-                                         const int ib[2], const T p[2], T c, FieldPt<T, 2> &F,
-                                         rev::RFrame<T, 2> &f)
+                                         const int ib[2], const T p[2], const StepPar<T> &s,
+                                         FieldPt<T, 2> &F, rev::RFrame<T, 2> &f)
 {
     if (pt < GCB_ADJ_FCACHE) fc.load(pt, F);
     else gather_any<T, 2, 2>(g, ib, p, F);
-    f.make(F, c);
+    f.make(F, s.c, s.inv_c2);
 }
 
 // Called by the whole warp (the additions to the node accumulators are made
@@ -573,7 +573,7 @@ __device__ __forceinline__ void gca_rev(const DevGrid<T> &g, NodeCache<T> &grad,
     T upn;
     if (on) {
         for (int j = 0; j < 2; ++j) {
-            frame_at(g, fc, j == 0 ? 1 : 0, ib, j == 0 ? pts[0] : l, s.c, F, f);
+            frame_at(g, fc, j == 0 ? 1 : 0, ib, j == 0 ? pts[0] : l, s, F, f);
             if (j == 0) rev::conv_fwd(f, s, u, cv);
             else upn = rev::upar_new(f, s, cv.upar, cv.mu, cv.uperp);
         }
@@ -593,7 +593,7 @@ __device__ __forceinline__ void gca_rev(const DevGrid<T> &g, NodeCache<T> &grad,
             const int pt = st == 0 ? K + 1 : (st < K ? K - st + 1 : (st == K ? 0 : 1));
             p[0] = q[0];
             p[1] = q[1];
-            frame_at(g, fc, pt, ib, p, s.c, F, f);
+            frame_at(g, fc, pt, ib, p, s, F, f);
             FrameAdj<T> af;
             af.zero();
             if (st == 0) {

@@ -38,9 +38,10 @@ __device__ __forceinline__ bool pos_finite(double x) { return !not_pos_normal(x)
 // one; FP32's hold |E x B|^2 for 1e-9 to 4e9 only.  There (F32) |v_E|^2 is taken
 // from v_E and every product of two fields meets its 1/|B| before the next
 // (lean_drift, the u_par update), which keeps all of them within |B|^2, good for
-// 1e-19 to 1e19 (from 1e-19 sqrt(c) up, c/|B|^2 being one of them).  It costs nothing worth having (GB300, 2^24 particles in 2D, 8
-// steps and their sort: one factor |B|^-3 8.18 ms, this 8.21; the order of
-// lean_drift's prefactor decides, with kappa^2 apart 8 B more spilled, 8.37).
+// 1e-19 to 1e19 (from 1e-19 sqrt(c) up, c/|B|^2 being one of them).  It costs
+// nothing worth having (GB300, 2^24 particles in 2D, 8 steps and their sort: one
+// factor |B|^-3 8.18 ms, this 8.21; the order of lean_drift's prefactor decides,
+// with kappa^2 apart 8 B more spilled, 8.37).
 template <typename R>
 struct LeanFrame {
     static constexpr bool F32 = sizeof(R) == 4;

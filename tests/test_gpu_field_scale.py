@@ -69,3 +69,28 @@ def test_push(G, kind, option, precision, k):
     bad |= (np.abs(a["u"] - b["u"]) > TOL * (1.0 + np.linalg.norm(a["u"], axis=0))).any(0)
     bad |= (np.abs(a["dxp"] - b["dxp"]) > TOL).any(0)
     assert bad.mean() < 1e-3
+
+
+@pytest.mark.parametrize("k", SCALES)
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_adjoint(G, precision, k):
+    """Gradients of the state as they are, those of the records by 2^-k."""
+    import torch
+    base, pats, amps, st, p = inputs.reconnection_2d_modes(
+        nx=64, ny=32, delta=2.0, n_modes=2, max_mode=2, n_particles=2003, omega_dt_max=50.0, seed=3)
+    fields = inputs.combine_fields(base, pats, amps)
+    res = []
+    for kk in (0, k):
+        f, q = scaled(fields, p, kk)
+        grid = G.Grid(f, dtype="f64" if precision == "fp64" else "f32")
+        ds = G.State.from_numpy(st, precision=precision, pos_mode="pair")
+        lam = torch.randn((7, ds.n), dtype=ds.u.dtype, device="cuda",
+                          generator=torch.Generator(device="cuda").manual_seed(5))
+        grad = G.adjoint(ds, grid, G.make_params(q, gca_fixed_iters=4), 2, lam, 2)
+        res.append((lam.double().cpu().numpy(), grad.cpu().numpy() * 2.0 ** kk))
+    for a, b in zip(*res):
+        ref = a if a.shape[0] == 7 else a.T
+        got = b if b.shape[0] == 7 else b.T
+        rms = np.sqrt((ref ** 2).mean(1, keepdims=True))
+        assert (rms > 0).all() and np.isfinite(got).all()
+        assert (np.abs(got - ref) > TOL * (np.abs(ref) + rms)).mean() < 1e-3
