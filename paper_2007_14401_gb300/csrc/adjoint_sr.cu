@@ -58,10 +58,12 @@ struct DualGather {
         D t[2];
 #pragma unroll
         for (int d = 0; d < 2; ++d) {
+            // cell and fraction from one rounding (cell_of's), with the
+            // position's tangent
             T tv;
             cell_of(g, d, ib[d], l[d].v, tv, i0[d], i1[d]);
-            const T c = floor(l[d].v * g.inv_dx[d]);
-            t[d] = l[d] * g.inv_dx[d] - c;   // = tv, with the position's tangent
+            t[d] = l[d] * g.inv_dx[d];
+            t[d].v = tv;
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) { F.E[c] = D(T(0)); F.B[c] = D(T(0)); }
