@@ -121,8 +121,7 @@ struct AdjArgs {
     double *grad;                // node records' adjoint, stride 12 per node
     StepPar<T> sp;
     T qm[4];
-    T rho_thr, f_E, c2;
-    int force;
+    Switch<T> sw;
 };
 
 template <typename T>
@@ -184,14 +183,8 @@ __global__ void __launch_bounds__(TPB) k_adjoint_sr(const AdjArgs<T> a)
         sp.qm = a.qm[(fl >> GCB_SPECIES_SHIFT) & 3];
         sp.cq = sp.c / sp.qm;
         FieldPt<T, 2> F0;
-        gather<T, 2, 2>(a.g, ib, l, F0);
-        const T Q = fabs(sp.qm);
-        const T G = sqrt(T(1) + (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * sp.inv_c2);
-        const T Bm = sqrt(F0.B[0] * F0.B[0] + F0.B[1] * F0.B[1] + F0.B[2] * F0.B[2]);
-        const T Em = sqrt(F0.E[0] * F0.E[0] + F0.E[1] * F0.E[1] + F0.E[2] * F0.E[2]);
-        int S = (a.c2 * G < a.rho_thr * Q * Bm && Em < a.f_E * Bm) ? 0 : 1;
-        if (a.force == GCB_FORCE_BORIS) S = 1;
-        if (a.force == GCB_FORCE_GCA) S = 0;
+        gather_any<T, 2, 2>(a.g, ib, l, F0);
+        const int S = a.sw(F0, u, sp.inv_c2, (fl >> GCB_SPECIES_SHIFT) & 3, a.qm);
         int iters = 0;
         bool gca = false;
         if (S == 0) {
@@ -701,13 +694,7 @@ __global__ void __launch_bounds__(TPB, RevBlocks<T>::n) k_adjoint_rev(const AdjA
             sp.cq = sp.c / sp.qm;
             gather_any<T, 2, 2>(a.g, ib, l, F0);
             fc.store(0, F0);
-            const T Q = fabs(sp.qm);
-            const T G = sqrt(T(1) + (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * sp.inv_c2);
-            const T Bm = sqrt(F0.B[0] * F0.B[0] + F0.B[1] * F0.B[1] + F0.B[2] * F0.B[2]);
-            const T Em = sqrt(F0.E[0] * F0.E[0] + F0.E[1] * F0.E[1] + F0.E[2] * F0.E[2]);
-            int S = (a.c2 * G < a.rho_thr * Q * Bm && Em < a.f_E * Bm) ? 0 : 1;
-            if (a.force == GCB_FORCE_BORIS) S = 1;
-            if (a.force == GCB_FORCE_GCA) S = 0;
+            const int S = a.sw(F0, u, sp.inv_c2, (fl >> GCB_SPECIES_SHIFT) & 3, a.qm);
             if (S == 0) {
                 T uu[3] = {u[0], u[1], u[2]}, disp[2];
                 bool ncv;
@@ -822,10 +809,7 @@ gcb_status adjoint_step(const gcb_particles *s, const gcb_grid *g, const gcb_par
         a.sp.fixed_iters = prm->gca_fixed_iters;
         a.sp.tol = (T)prm->gca_tol;
         for (int k = 0; k < 4; ++k) a.qm[k] = (T)prm->qm[k];
-        a.rho_thr = (T)(prm->f_rho * prm->dl);
-        a.f_E = (T)prm->f_E;
-        a.c2 = (T)(prm->c * prm->c);
-        a.force = prm->force;
+        a.sw.fill(prm);
     };
     if (s->mom_dtype == GCB_F64) {
         adj::AdjArgs<double> a;

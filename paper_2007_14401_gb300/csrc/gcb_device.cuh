@@ -10,11 +10,13 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <climits>
 #include <type_traits>
 
+#include "gcb.h"
 #include "real64.cuh"
 
 namespace gcb {
@@ -729,6 +731,52 @@ struct StepPar {
     int curvature, mu_mode, max_iter, fixed_iters;
     R tol;
     int phase;   // 1: the gyration phase advances over the step (GCB_PHASE_EVOLVE)
+};
+
+// The switch S (Sec. 3, Sec. 4.1) in division-free form: S = 0 iff c^2 Gamma <
+// f_rho dl |q/m| B and |E| < f_E B.  One place for the push and for the adjoint's
+// replay, which has to find the branch that the push took also for a particle
+// within rounding of the threshold.
+template <typename R>
+struct Switch {
+    double w2[4], f_E2;       // FP64: (f_rho dl |q/m|/c^2)^2 and f_E^2
+    R rho_thr, f_E, c2;       // FP32: f_rho dl, f_E and c^2
+    int force;
+
+    void fill(const gcb_params *prm)
+    {
+        for (int k = 0; k < 4; ++k) {
+            const double w = prm->f_rho * prm->dl * fabs(prm->qm[k]) / (prm->c * prm->c);
+            w2[k] = w * w;
+        }
+        f_E2 = prm->f_E * prm->f_E;
+        rho_thr = (R)(prm->f_rho * prm->dl);
+        f_E = (R)prm->f_E;
+        c2 = (R)(prm->c * prm->c);
+        force = prm->force;
+    }
+    // S of a particle of species sp with momentum u where the fields are F
+    template <int ND>
+    __device__ __forceinline__ int operator()(const FieldPt<R, ND> &F, const R u[3], R inv_c2, int sp,
+                                              const R qm[4]) const
+    {
+        int S;
+        if constexpr (sizeof(R) == 8) {
+            // squared: no roots (each ~10 FP64 operations)
+            const double G2 = fma(dot3(u, u), inv_c2, 1.0);
+            const double B2 = dot3(F.B, F.B), E2 = dot3(F.E, F.E);
+            S = (G2 < w2[sp] * B2 && E2 < f_E2 * B2) ? 0 : 1;
+        } else {
+            const R Q = fabs(qm[sp]);
+            const R G = sqrt(R(1) + dot3(u, u) * inv_c2);
+            const R Bm = sqrt(dot3(F.B, F.B));
+            const R Em = sqrt(dot3(F.E, F.E));
+            S = (c2 * G < rho_thr * Q * Bm && Em < f_E * Bm) ? 0 : 1;
+        }
+        if (force == GCB_FORCE_BORIS) S = 1;
+        if (force == GCB_FORCE_GCA) S = 0;
+        return S;
+    }
 };
 
 // Gyration energy term of Eq. (lfacgca2): 2 mu B kappa / m, or u_perp,g^2

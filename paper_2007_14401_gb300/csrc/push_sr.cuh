@@ -98,11 +98,7 @@ struct PushArgs {
     int64_t *pid;             // written only when pidin differs
     StepPar<R> sp;            // sp.qm and sp.cq are set per particle
     R qm[4], cq[4];           // per species: q/m and c/(q/m)
-    double sw[4], f_E2;       // FP64 switch: (f_rho dl |q/m|/c^2)^2 and f_E^2
-    R rho_thr;                // f_rho * dl
-    R f_E;
-    R c2;
-    int force;
+    Switch<R> sw;
     int nsteps;               // steps of this launch (> 1 only for the fused kernel)
     unsigned long long *stats;
     // current deposition (kernels with DEP)
@@ -468,24 +464,7 @@ __global__ void __launch_bounds__(Tile<R, ND>::n, MinBlocks<R, ND, GM, DEP, BT>:
                 }
                 if constexpr (GCB_SEED_CACHE && Gth::kCellCache) gather_cached<ND, GM>(a.g, ib, l, F, cr);
                 else Gth{a.g}(ib, l, F);
-                // switch S (Sec. 3, Sec. 4.1) in division-free form:
-                // S = 0 iff c^2 Gamma < f_rho dl |q/m| B and |E| < f_E B.
-                int S;
-                if constexpr (sizeof(R) == 8) {
-                    // squared: no roots (each ~10 FP64 operations)
-                    const double G2 = fma(dot3(uu, uu), a.sp.inv_c2, 1.0);
-                    const double B2 = dot3(F.B, F.B), E2 = dot3(F.E, F.E);
-                    S = (G2 < a.sw[(fl >> GCB_SPECIES_SHIFT) & 3] * B2 && E2 < a.f_E2 * B2) ? 0 : 1;
-                } else {
-                    R Q = fabs(a.qm[(fl >> GCB_SPECIES_SHIFT) & 3]);
-                    R G = sqrt(R(1) + dot3(uu, uu) * a.sp.inv_c2);
-                    R Bm = sqrt(dot3(F.B, F.B));
-                    R Em = sqrt(dot3(F.E, F.E));
-                    S = (a.c2 * G < a.rho_thr * Q * Bm && Em < a.f_E * Bm) ? 0 : 1;
-                }
-                if (a.force == GCB_FORCE_BORIS) S = 1;
-                if (a.force == GCB_FORCE_GCA) S = 0;
-                cls = S;
+                cls = a.sw(F, uu, a.sp.inv_c2, (fl >> GCB_SPECIES_SHIFT) & 3, a.qm);
             } else {
                 // frozen: written back unchanged (with its flag) right here;
                 // fused, it stays in its slot for the final store
@@ -850,14 +829,8 @@ static void fill_args(PushArgs<R> &a, const gcb_particles *p, const gcb_particle
     for (int k = 0; k < 4; ++k) {
         a.qm[k] = (R)prm->qm[k];
         a.cq[k] = a.sp.c / a.qm[k];
-        const double w = prm->f_rho * prm->dl * fabs(prm->qm[k]) / (prm->c * prm->c);
-        a.sw[k] = w * w;
     }
-    a.f_E2 = prm->f_E * prm->f_E;
-    a.rho_thr = (R)(prm->f_rho * prm->dl);
-    a.f_E = (R)prm->f_E;
-    a.c2 = (R)(prm->c * prm->c);
-    a.force = prm->force;
+    a.sw.fill(prm);
     a.nsteps = 1;
     a.stats = stats;
 }
