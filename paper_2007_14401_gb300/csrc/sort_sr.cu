@@ -91,6 +91,7 @@ static int caller_arrays(const gcb_particles *p, int ndim, void **a)
 struct KeyArgs {
     int64_t n;
     const void *x[3];
+    const float *xlo[3];   // FP32-pair positions (PosT float)
     float inv_dx[3];
     int ncell[3], tile[3], ntile[3];
     int32_t *keys, *ranks, *hist;
@@ -101,8 +102,9 @@ struct KeyArgs {
 // returns: four particles a thread keep four of each in flight.  Runs of equal
 // keys are found from the neighbouring lane; a match over the whole warp merges
 // a few more lanes but was what the kernel waited for.  FP32-pair positions:
-// the high parts alone decide the cell.  Measured (GB300): 2^24 particles 2D 235
-// -> 63 us, 3D 247 -> 89 us, 2^20 20 -> 7 us.
+// the high parts decide the cell, the low ones are read because either part may
+// be what is not finite.  Measured (GB300): 2^24 particles 3D 247 -> 116 us (84
+// with the high parts alone), 2^20 2D 20 -> 6.4 us (5.4).
 constexpr int kKeyItems = 4;
 template <typename PosT, int ND>
 __global__ void __launch_bounds__(256) k_sort_keys(const KeyArgs a)
@@ -118,6 +120,11 @@ __global__ void __launch_bounds__(256) k_sort_keys(const KeyArgs a)
 #pragma unroll
             for (int d = 0; d < ND; ++d)
                 x[j][d] = i < a.n ? static_cast<const PosT *>(a.x[d])[i] : PosT(0);
+            if constexpr (sizeof(PosT) == 4) {
+#pragma unroll
+                for (int d = 0; d < ND; ++d)   // hi, or NaN where lo is not finite
+                    x[j][d] = fmaf(0.0f, i < a.n ? a.xlo[d][i] : 0.0f, x[j][d]);
+            }
         }
 #pragma unroll
         for (int j = 0; j < kKeyItems; ++j) {
@@ -403,6 +410,7 @@ gcb_status sort_into_workspace(const gcb_particles *p, const gcb_grid *g, const 
     ka.n = p->n;
     for (int d = 0; d < 3; ++d) {
         ka.x[d] = p->x[d];
+        ka.xlo[d] = static_cast<const float *>(p->x_lo[d]);
         ka.inv_dx[d] = (float)(1.0 / g->dx[d]);
         ka.ncell[d] = (int)g->n[d];
         ka.tile[d] = pl.tile[d];
