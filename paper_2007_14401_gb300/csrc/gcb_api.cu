@@ -573,6 +573,23 @@ static gcb_status push_sr_impl(const gcb_particles *p, const gcb_grid *g, const 
         set_error("cudaMemsetAsync: %s", cudaGetErrorString(cudaGetLastError()));
         return GCB_ECUDA;
     }
+    // a call with statistics also readies the kernels that the same steps without
+    // them run (an empty set: sized and loaded, not launched), those of one step a
+    // launch and, where steps are fused, of several, so that a program that has
+    // pushed once may capture pushes into a graph
+    gcb_particles none = *p;
+    none.n = 0;
+    for (int k = 1; stats && n_steps > 0 && s == GCB_OK;) {
+        if (cur)
+            s = (fp64 ? push_dep_step_f64_quiet : push_dep_step_f32_quiet)(&none, &none, g, prm, cur, st, nullptr);
+        else if (prm->mirror == GCB_MIRROR_ON)
+            s = (fp64 ? push_mir_step_f64_quiet : push_mir_step_f32_quiet)(&none, &none, g, prm, st, nullptr);
+        else
+            s = (fp64 ? push_step_f64_quiet : push_step_f32_quiet)(&none, &none, g, prm, st, nullptr, k);
+        if (k >= prm->fuse_steps) break;
+        k = prm->fuse_steps;
+    }
+    if (s != GCB_OK) return s;
     for (int step = 0; step < n_steps;) {
         const gcb_particles *in = p;
         gcb_particles q;
@@ -594,27 +611,18 @@ static gcb_status push_sr_impl(const gcb_particles *p, const gcb_grid *g, const 
                 k = k < to_sort ? k : to_sort;
             }
         }
-        // a call with statistics also readies the kernel that a call without
-        // runs (an empty set: sized and loaded, not launched), so that a program
-        // that has pushed once may capture pushes into a graph
-        gcb_particles none = *p;
-        none.n = 0;
-        const bool ready = stats && step == 0;
         if (cur) {
             auto fn = fp64 ? (stats ? push_dep_step_f64 : push_dep_step_f64_quiet)
                            : (stats ? push_dep_step_f32 : push_dep_step_f32_quiet);
-            if (ready) s = (fp64 ? push_dep_step_f64_quiet : push_dep_step_f32_quiet)(&none, &none, g, prm, cur, st, nullptr);
-            if (s == GCB_OK) s = fn(p, in, g, prm, cur, st, stats);
+            s = fn(p, in, g, prm, cur, st, stats);
         } else if (prm->mirror == GCB_MIRROR_ON) {
             auto fn = fp64 ? (stats ? push_mir_step_f64 : push_mir_step_f64_quiet)
                            : (stats ? push_mir_step_f32 : push_mir_step_f32_quiet);
-            if (ready) s = (fp64 ? push_mir_step_f64_quiet : push_mir_step_f32_quiet)(&none, &none, g, prm, st, nullptr);
-            if (s == GCB_OK) s = fn(p, in, g, prm, st, stats);
+            s = fn(p, in, g, prm, st, stats);
         } else {
             auto fn = fp64 ? (stats ? push_step_f64 : push_step_f64_quiet)
                            : (stats ? push_step_f32 : push_step_f32_quiet);
-            if (ready) s = (fp64 ? push_step_f64_quiet : push_step_f32_quiet)(&none, &none, g, prm, st, nullptr, k);
-            if (s == GCB_OK) s = fn(p, in, g, prm, st, stats, k);
+            s = fn(p, in, g, prm, st, stats, k);
         }
         if (s != GCB_OK) return s;
         step += k;
@@ -886,6 +894,13 @@ gcb_status gcb_push_sr_ckpt(const gcb_particles *p, const gcb_grid *g, const gcb
                 return (stats ? push_step_f64 : push_step_f64_quiet)(out_p, in, g, &prm, st, stats, 1);
             return (stats ? push_step_adj_f32 : push_step_adj_f32_quiet)(out_p, in, g, &prm, st, stats);
         };
+        if (stats) {   // the kernel without statistics readied too (see push_sr_impl)
+            gcb_particles none = *p;
+            none.n = 0;
+            s = fp64 ? push_step_f64_quiet(&none, &none, g, &prm, st, nullptr, 1)
+                     : push_step_adj_f32_quiet(&none, &none, g, &prm, st, nullptr);
+            if (s != GCB_OK) return s;
+        }
         // with sorting the last step writes here, the source of the final permutation
         gcb_particles t = state_view(p, nd, w + L.tmp);
         if (L.sort && p->pid) t.pid = (int64_t *)(w + L.pidt);
