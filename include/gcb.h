@@ -385,6 +385,20 @@ gcb_status gcb_adjoint_sr(const gcb_particles *p0, const gcb_grid *g, const gcb_
                           double *grad_rec, void *cuda_stream, void *ws, size_t ws_bytes);
 
 /*
+ * gcb_push_sr with the step that gcb_adjoint_sr differentiates: the forward pass
+ * whose states a gcb_adjoint_sr without GCB_ADJ_HAVE_CKPT runs through, bit for
+ * bit.  In the mixed path gcb_push_sr takes that step in another order of
+ * operations (shorter, to which the adjoint's replay is not tied): its states
+ * differ from these by FP32 rounding at every step.  FP64: the same as
+ * gcb_push_sr.  Arguments and errors as gcb_push_sr (what the adjoint does not
+ * differentiate is pushed as there; fuse_steps does not apply to the mixed
+ * path's 2D gradient-record step).
+ */
+gcb_status gcb_push_sr_adj(const gcb_particles *p, const gcb_grid *g, const gcb_params *prm,
+                           int n_steps, void *cuda_stream, void *ws, size_t ws_bytes,
+                           gcb_stats *out);
+
+/*
  * The forward pass for a later gcb_adjoint_sr: n_steps pushes of p in place
  * that also store, in the adjoint workspace ws, the initial state and every
  * ckpt_every-th state (sorted by cell first when prm->sort_every > 0; p then

@@ -534,12 +534,19 @@ static gcb_status check_current(const gcb_particles *p, const gcb_grid *g, const
 
 static gcb_status push_sr_impl(const gcb_particles *p, const gcb_grid *g, const gcb_params *prm,
                                const gcb_current *cur, int n_steps, void *cuda_stream, void *ws,
-                               size_t ws_bytes, gcb_stats *out, gcb_deposit_stats *dst);
+                               size_t ws_bytes, gcb_stats *out, gcb_deposit_stats *dst,
+                               bool as_adjoint = false);
 
 gcb_status gcb_push_sr(const gcb_particles *p, const gcb_grid *g, const gcb_params *prm,
                        int n_steps, void *cuda_stream, void *ws, size_t ws_bytes, gcb_stats *out)
 {
     return push_sr_impl(p, g, prm, nullptr, n_steps, cuda_stream, ws, ws_bytes, out, nullptr);
+}
+
+gcb_status gcb_push_sr_adj(const gcb_particles *p, const gcb_grid *g, const gcb_params *prm,
+                           int n_steps, void *cuda_stream, void *ws, size_t ws_bytes, gcb_stats *out)
+{
+    return push_sr_impl(p, g, prm, nullptr, n_steps, cuda_stream, ws, ws_bytes, out, nullptr, true);
 }
 
 gcb_status gcb_push_deposit_sr(const gcb_particles *p, const gcb_grid *g, const gcb_params *prm,
@@ -551,9 +558,13 @@ gcb_status gcb_push_deposit_sr(const gcb_particles *p, const gcb_grid *g, const 
     return push_sr_impl(p, g, prm, cur, n_steps, cuda_stream, ws, ws_bytes, out, dst);
 }
 
+// as_adjoint: the step that the adjoint's forward run takes, where that is
+// another than the push's own (mixed path, 2D, gradient records, the options that
+// the adjoint differentiates)
 static gcb_status push_sr_impl(const gcb_particles *p, const gcb_grid *g, const gcb_params *prm,
                                const gcb_current *cur, int n_steps, void *cuda_stream, void *ws,
-                               size_t ws_bytes, gcb_stats *out, gcb_deposit_stats *dst)
+                               size_t ws_bytes, gcb_stats *out, gcb_deposit_stats *dst,
+                               bool as_adjoint)
 {
     g_err[0] = 0;
     gcb_status s = check_problem(p, g, prm);
@@ -566,6 +577,10 @@ static gcb_status push_sr_impl(const gcb_particles *p, const gcb_grid *g, const 
     if (!ws || !aligned(ws, 256)) { set_error("workspace NULL or not 256-byte aligned"); return GCB_EINVAL; }
     if (ws_bytes < kStatsBytes) { set_error("workspace too small"); return GCB_ENOMEM; }
     const bool fp64 = p->mom_dtype == GCB_F64;
+    const bool adj = as_adjoint && !fp64 && g->ndim == 2 && prm->grad_mode == GCB_GRAD_GRID &&
+                     prm->drift_frame == GCB_FRAME_SIMPLE && prm->gyro_phase == GCB_PHASE_KEEP &&
+                     prm->mirror == GCB_MIRROR_OFF;
+    const int fuse = adj ? 1 : prm->fuse_steps;   // that step has no fused kernel
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
     unsigned long long *stats = out || dst ? (unsigned long long *)ws : nullptr;
@@ -584,10 +599,12 @@ static gcb_status push_sr_impl(const gcb_particles *p, const gcb_grid *g, const 
             s = (fp64 ? push_dep_step_f64_quiet : push_dep_step_f32_quiet)(&none, &none, g, prm, cur, st, nullptr);
         else if (prm->mirror == GCB_MIRROR_ON)
             s = (fp64 ? push_mir_step_f64_quiet : push_mir_step_f32_quiet)(&none, &none, g, prm, st, nullptr);
+        else if (adj)
+            s = push_step_adj_f32_quiet(&none, &none, g, prm, st, nullptr);
         else
             s = (fp64 ? push_step_f64_quiet : push_step_f32_quiet)(&none, &none, g, prm, st, nullptr, k);
-        if (k >= prm->fuse_steps) break;
-        k = prm->fuse_steps;
+        if (k >= fuse) break;
+        k = fuse;
     }
     if (s != GCB_OK) return s;
     for (int step = 0; step < n_steps;) {
@@ -604,8 +621,8 @@ static gcb_status push_sr_impl(const gcb_particles *p, const gcb_grid *g, const 
         // steps fused into this launch: at most fuse_steps, none past the
         // next sort
         int k = 1;
-        if (prm->fuse_steps > 1) {
-            k = prm->fuse_steps < n_steps - step ? prm->fuse_steps : n_steps - step;
+        if (fuse > 1) {
+            k = fuse < n_steps - step ? fuse : n_steps - step;
             if (prm->sort_every > 0) {
                 const int to_sort = prm->sort_every - (int)(gstep % prm->sort_every);
                 k = k < to_sort ? k : to_sort;
@@ -619,6 +636,8 @@ static gcb_status push_sr_impl(const gcb_particles *p, const gcb_grid *g, const 
             auto fn = fp64 ? (stats ? push_mir_step_f64 : push_mir_step_f64_quiet)
                            : (stats ? push_mir_step_f32 : push_mir_step_f32_quiet);
             s = fn(p, in, g, prm, st, stats);
+        } else if (adj) {
+            s = (stats ? push_step_adj_f32 : push_step_adj_f32_quiet)(p, in, g, prm, st, stats);
         } else {
             auto fn = fp64 ? (stats ? push_step_f64 : push_step_f64_quiet)
                            : (stats ? push_step_f32 : push_step_f32_quiet);

@@ -85,8 +85,8 @@ DEPOSIT_MAX_CELLS = 64   # GCB_DEPOSIT_MAX_CELLS
 EXPORTS = ["gcb_version", "gcb_status_string", "gcb_last_error", "gcb_grid_stride",
            "gcb_grid_pack", "gcb_pos_split", "gcb_pos_join", "gcb_workspace_bytes",
            "gcb_sort_sr", "gcb_push_sr", "gcb_push_sr_noalloc", "gcb_adjoint_workspace_bytes",
-           "gcb_adjoint_sr", "gcb_push_sr_ckpt", "gcb_grid_combine", "gcb_grad_project", "gcb_ks_cell_size",
-           "gcb_push_ks", "gcb_push_deposit_sr"]
+           "gcb_adjoint_sr", "gcb_push_sr_adj", "gcb_push_sr_ckpt", "gcb_grid_combine",
+           "gcb_grad_project", "gcb_ks_cell_size", "gcb_push_ks", "gcb_push_deposit_sr"]
 
 
 def load_library(path: str | None = None):
@@ -113,6 +113,8 @@ def load_library(path: str | None = None):
     lib.gcb_push_sr.argtypes = [P(GcbParticles), P(GcbGrid), P(GcbParams), C.c_int,
                                 C.c_void_p, C.c_void_p, C.c_size_t, P(GcbStats)]
     lib.gcb_push_sr.restype = C.c_int
+    lib.gcb_push_sr_adj.argtypes = lib.gcb_push_sr.argtypes
+    lib.gcb_push_sr_adj.restype = C.c_int
     lib.gcb_sort_sr.argtypes = [P(GcbParticles), P(GcbGrid), P(GcbParams), C.c_void_p,
                                 C.c_void_p, C.c_size_t]
     lib.gcb_sort_sr.restype = C.c_int
@@ -566,6 +568,18 @@ class AdjointWorkspace:
         self.have_ckpt = False
 
 
+def push_adj(state: State, grid: Grid, params: GcbParams, n_steps: int, stream=None,
+             workspace: Workspace | None = None):
+    """n_steps pushes of ``state`` in place through the states that a following
+    adjoint(..., workspace=None) from the same start differentiates, bit for bit.
+    (push itself takes the mixed path's step in another order of operations, so
+    that its states differ from these by FP32 rounding; in FP64 they are equal.)"""
+    ws = workspace or Workspace(state, grid, params, _work_device(state))
+    rc = _lib.gcb_push_sr_adj(C.byref(state.s), C.byref(grid.s), C.byref(params), int(n_steps),
+                              _stream_ptr(stream), C.c_void_p(ws.buf.data_ptr()), ws.nbytes, None)
+    _check(rc, "gcb_push_sr_adj")
+
+
 def push_ckpt(state: State, grid: Grid, params: GcbParams, n_steps: int,
               workspace: AdjointWorkspace, stream=None, stats: bool = False):
     """n_steps pushes of ``state`` in place that also store the adjoint's
@@ -591,7 +605,8 @@ def adjoint(state: State, grid: Grid, params: GcbParams, n_steps: int, lam: torc
     Returns dL/d(record values) as a float64 tensor (nodes, 12).  method
     "reverse" (default) or "tangent" (dual-number Jacobian columns, slower).
     A ``workspace`` filled by push_ckpt supplies the checkpoints (and its
-    n_steps / ckpt_every must match); otherwise the forward is rerun here."""
+    n_steps / ckpt_every must match); otherwise the forward is rerun here, as
+    push_adj takes it (in the mixed path push differs from it by rounding)."""
     if workspace is None:
         workspace = AdjointWorkspace(state, grid, n_steps, ckpt_every, params)
     elif (workspace.n_steps, workspace.ckpt_every) != (int(n_steps), int(ckpt_every)):
@@ -659,7 +674,7 @@ class ModePush(torch.autograd.Function):
             # (the adjoint sorts at its checkpoints and restores the order)
             fwd = GcbParams.from_buffer_copy(cfg["params"])
             fwd.sort_every = 0
-            push(st, grid, fwd, cfg["n_steps"], stats=False)
+            push_adj(st, grid, fwd, cfg["n_steps"])
         return st.x_f64(), st.u.clone(), st.dxp.clone()
 
     @staticmethod
