@@ -877,20 +877,16 @@ __device__ __forceinline__ void boris(const R E[3], const R B[3], const StepPar<
 // records of the last cell it loaded in cr (FP32: CellRecs); the step then
 // passes every gather after the one at x^n through it.
 // Which FP32 kernels keep the cell's records between gathers: measured on
-// GB300, the 3D push (8 nodes of 2 record chunks per gather) gains 9%, the
-// 2D push with gradient records (4 nodes of 3 chunks) loses 2-4% to the
-// registers the records take.
-#ifndef GCB_CELL_CACHE_2D
-#define GCB_CELL_CACHE_2D 0
-#endif
+// GB300, the 3D push (8 nodes of 2 record chunks per gather) gains 9%; the
+// 2D push with gradient records (4 nodes of 3 chunks) lost 2-4% to the
+// registers the records take, so that 2D has none (nor has gca_lean.cuh).
 #ifndef GCB_CELL_CACHE_3D
 #define GCB_CELL_CACHE_3D 1
 #endif
 // RAW: shape-function gradients left per cell (FP64, see RawGrad).
 template <typename R, int ND, int GM, bool RAW = false>
 struct PlainGather {
-    static constexpr bool kCellCache =
-        sizeof(R) == 4 && (ND == 2 ? GCB_CELL_CACHE_2D : GCB_CELL_CACHE_3D);
+    static constexpr bool kCellCache = sizeof(R) == 4 && ND == 3 && GCB_CELL_CACHE_3D;
     DevGrid<R> g;
     __device__ __forceinline__ void operator()(const int ib[ND], const R l[ND],
                                                FieldPt<R, ND> &F) const
