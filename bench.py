@@ -521,7 +521,8 @@ def run_reference(args, rank, w):
 
 
 # Kernels of one sort on this file's grids: keys, two of the scan, inverse,
-# gather (past 2^25 buckets the scan has a third, 6 in all).
+# gather.  Past 2^25 buckets the scan has a third, 6 in all, which is what
+# fused_launches and adjoint_launches take when they are not told.
 SORT_KERNELS = 5
 
 

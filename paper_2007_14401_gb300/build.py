@@ -28,9 +28,11 @@ SOURCES = ["gcb_api.cu", "sort_sr.cu", "gcb_noalloc.cu", "gcb_ks.cu", "adjoint_s
 SOURCES += [s.replace(".cu", "_quiet.cu") for s in SOURCES if s.startswith("push_")]
 # The mixed-precision push and the adjoint unit use approximate FP32 division
 # and square root (about 2 ulp) and flush FP32 denormals: the flags act on
-# single precision only, so the FP64 kernels in the adjoint unit keep IEEE
-# operations, as does the FP64 push.  The adjoint's FP32 replay of a step then
-# uses the same arithmetic as the FP32 push it retraces.
+# single precision only.  The FP64 kernels compile as everywhere; their
+# reciprocals and roots are those of csrc/real64.cuh (within 1 ulp, the root 2;
+# denormal arguments count as 0, denormal results are flushed) where that file's
+# functions are called, else IEEE.  The adjoint's FP32 replay of a step then
+# uses the same arithmetic as the FP32 forward run it retraces.
 EXTRA = {"push_sr_f32.cu": ["-use_fast_math"], "push_dep_f32.cu": ["-use_fast_math"],
          "push_mir_f32.cu": ["-use_fast_math"],
          "adjoint_sr.cu": ["-use_fast_math"]}

@@ -239,7 +239,8 @@ __device__ __forceinline__ void gc_vel_bwd(const F &f, const StepPar<T> &s, T up
 template <typename T>
 struct Quad { T A, gg, D, iD, upr, P0, k1, k2, G1, upn; Gam<T> g0; };
 
-// (rG: the root chosen as the forward step does, the larger of the two)
+// (of k1 G^2 + k2 G + k3 = 0 with k1 < 0 < k3 the one positive root, as in the
+// forward step)
 template <typename T, typename F>
 __device__ __forceinline__ void quad_r(const F &f0, const StepPar<T> &s, T upar, T mu, T uperp, Quad<T> &q)
 {
