@@ -39,9 +39,10 @@ __device__ __forceinline__ bool pos_finite(double x) { return !not_pos_normal(x)
 // from v_E and every product of two fields meets its 1/|B| before the next
 // (lean_drift, the u_par update), which keeps all of them within |B|^2, good for
 // 1e-19 to 1e19 (from 1e-19 sqrt(c) up, c/|B|^2 being one of them).  It costs
-// nothing worth having (GB300, 2^24 particles in 2D, 8 steps and their sort: one
-// factor |B|^-3 8.18 ms, this 8.21; the order of lean_drift's prefactor decides,
-// with kappa^2 apart 8 B more spilled, 8.37).
+// (GB300, 2D, against one factor |B|^-3) 7 of 1358 instructions a particle-step:
+// 2^24 particles, 8 steps and their sort 8.18 -> 8.21 ms; 8 steps of 3000017
+// particles in one launch 1.45 -> 1.48 ms.  The order of lean_drift's prefactor
+// matters: with kappa^2 apart 8 B more are spilled, 8.37 ms.
 template <typename R>
 struct LeanFrame {
     static constexpr bool F32 = sizeof(R) == 4;

@@ -103,8 +103,8 @@ struct KeyArgs {
 // keys are found from the neighbouring lane; a match over the whole warp merges
 // a few more lanes but was what the kernel waited for.  FP32-pair positions:
 // the high parts decide the cell, the low ones are read because either part may
-// be what is not finite.  Measured (GB300): 2^24 particles 3D 247 -> 116 us (84
-// with the high parts alone), 2^20 2D 20 -> 6.4 us (5.4).
+// be what is not finite.  Measured (GB300): 2^24 particles 2D 235 -> 74 us (63
+// with the high parts alone), 3D 247 -> 116 us (84), 2^20 2D 20 -> 6.2 us (5.4).
 constexpr int kKeyItems = 4;
 template <typename PosT, int ND>
 __global__ void __launch_bounds__(256) k_sort_keys(const KeyArgs a)
