@@ -74,7 +74,9 @@ enum {
  * where the gradient block (3*ndim elements) is present iff has_grad, and
  * the stride (gcb_grid_stride) pads the record to a multiple of 16 bytes.
  * In 2D (ndim = 2) z is ignorable: positions have two components and
- * d_z = 0.  Build records with gcb_grid_pack.
+ * d_z = 0.  Build records with gcb_grid_pack.  The unit of the fields (and with
+ * it that of q/m) is the caller's: in FP32 squares of field values are formed,
+ * so |B| of about 1e-18 to 1e18.
  */
 typedef struct {
     int32_t ndim;            /* 2 or 3 */
